@@ -56,6 +56,16 @@ int phast_build_desc(const phast_system* sys, const phast_ff* ff, const phast_mu
         return phast_set_error(PHAST_EINVAL, "%s: box_L must be finite and >= 0", what);
     d->box_L = sys->box_L;
     d->inv_L = sys->box_L > 0.0 ? 1.0 / sys->box_L : 0.0;
+    d->img_lo = d->img_hi = 0x7fffffff;
+    if (sys->box_L > 0.0) {
+        auto high_word = [](double x) {
+            uint64_t b;
+            memcpy(&b, &x, sizeof(b));
+            return (int32_t)(b >> 32);
+        };
+        d->img_lo = high_word(0.5 * sys->box_L);
+        d->img_hi = high_word(1.5 * sys->box_L) - 1;
+    }
     if (!(sys->sphere_R >= 0.0) || !isfinite(sys->sphere_R))
         return phast_set_error(PHAST_EINVAL, "%s: sphere_R must be finite and >= 0", what);
     if (sys->sphere_R > 0.0 && sys->box_L > 0.0)

@@ -31,7 +31,8 @@ int phast_set_error(int code, const char* fmt, ...);
 struct SysDesc {
     int32_t n_chains, N, n_bins, recompute_every;
     int32_t walker_off, n_walkers, lnw_off, max_chain;
-    int32_t pair_precision, n_tiles, tile_off, pad0;
+    int32_t pair_precision, n_tiles, tile_off;
+    int32_t img_lo;       // high word of box_L / 2 (0x7fffffff: open space), see mimage64_short
     int64_t xyz_off;      // offset of walker 0's coordinates in the concatenated xyz (doubles)
     int64_t hw_off;       // offset of walker 0's histogram in hist_walker (bins)
     double box_L, inv_L;  // inv_L = 0 for open systems
@@ -41,7 +42,8 @@ struct SysDesc {
     double p[PHAST_N_MOVES], amax[PHAST_N_MOVES];
     uint64_t thr[PHAST_N_MOVES];   // move-type thresholds: type i if 2n+1 < thr[i] (n the 52-bit uniform), see propose_select
     int32_t last_type, type_mask;   // type_mask: bit i set when p[i] > 0
-    int32_t has_sphere, pad2;       // has_sphere: a steric container (sphere_R2 > 0)
+    int32_t has_sphere;             // a steric container (sphere_R2 > 0)
+    int32_t img_hi;                 // just below the high word of 3 box_L / 2 (0x7fffffff: open space)
     double sphere_R2;     // sphere_R * sphere_R of the steric container (0: none)
     double k_fene, fene_r0, fene_R, fene_kR2;   // FENE term of Eq. 2; fene_kR2 = k_fene * (R * R)
     double C_F[4];
@@ -301,6 +303,15 @@ __device__ __forceinline__ int bin_of(const SysDesc& d, double E) {
     return (int)floor(q);
 }
 
+// bin_of, the division by the bin width taken only where an FP32 estimate of the
+// quotient (error under 2e-7 of it) lies within its error of a bin edge.
+__device__ __forceinline__ int bin_of_short(const SysDesc& d, double E) {
+    const float x = (float)xsub(E, d.e_min) * d.iw32;
+    const float fl = floorf(x), fr = x - fl, mg = 4e-7f * fabsf(x) + 1e-6f;
+    if (fr > mg && fr < 1.0f - mg) return (fl < 0.0f || fl >= (float)d.n_bins) ? -1 : (int)fl;
+    return bin_of(d, E);
+}
+
 // ---------------------------------------------------------------------------
 // FP64 local terms.  Positions come from a functor pos(j) -> double3.
 // ---------------------------------------------------------------------------
@@ -401,6 +412,48 @@ __device__ __forceinline__ double lj64(double r2, double C) {
 // Minimum-image component (FP64); inv_L = 0 leaves d unchanged.
 __device__ __forceinline__ double mimage64(double dx, double L, double inv_L) {
     return dx - L * rint(dx * inv_L);
+}
+
+// The minimum image of mimage64, bit for bit, decided by the high word of dx (FP64
+// instructions hold the pipe for 64 cycles each on this chip, integer ones for one): a
+// word below that of L/2 means an image count of 0 (dx itself), one above it and clearly
+// below 3L/2 a count of +-1 (one addition: L is exact, so the fused product is too); the
+// rest takes mimage64.
+__device__ __forceinline__ double mimage64_short(const SysDesc& d, double dx) {
+    const int h = __double2hiint(dx) & 0x7fffffff;
+    if (h < d.img_lo) return dx;
+    if (h > d.img_lo && h < d.img_hi) return __dsub_rn(dx, copysign(d.box_L, dx));
+    return mimage64(dx, d.box_L, d.inv_L);
+}
+
+// 1/x and 1/sqrt(x) in FP64 from the hardware's approximations (relative error e0 of
+// about 2^-20) by one step of the series of 1/(1 - e) and (1 - e)^(-1/2), e the residual
+// of the approximation by fused multiply-adds: the truncated term is of order e0^3, far
+// below a rounding, so the result is within one rounding (rcp64) or two (rsqrt64) of the
+// true value, for 3 and 5 FP64 instructions instead of the 5.5 and 15 of 1.0/x and
+// 1.0/(sqrt(x) sqrt(y)).  Arguments whose approximation leaves the normal range (zero,
+// subnormal, huge, infinite, NaN, negative) take the plain operations.
+static __device__ __noinline__ double rcp64_plain(double x) { return 1.0 / x; }
+static __device__ __noinline__ double rsqrt64_plain(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ bool approx64_unsafe(double x) {
+    return (unsigned)__double2hiint(x) - 0x00200000u >= 0x7fa00000u;
+}
+__device__ __forceinline__ double rcp64(double x) {
+    if (approx64_unsafe(x)) return rcp64_plain(x);
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+__device__ __forceinline__ double rsqrt64(double x) {
+    if (approx64_unsafe(x)) return rsqrt64_plain(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
+}
+__device__ __forceinline__ double flip_sign(double x, bool flip) {
+    return __hiloint2double(__double2hiint(x) ^ (flip ? (int)0x80000000 : 0), __double2loint(x));
 }
 
 // Block-wide FP64 sum; every thread gets the result.  red: >= 32 doubles of shared.

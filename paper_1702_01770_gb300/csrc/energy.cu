@@ -72,11 +72,11 @@ delta_kernel(const SysDesc d, int B, const double* __restrict__ xyz, const phast
     const bool wall = ok && !container_ok<32, PT>(d, const_cast<double*>(x64), P, M, s, g, true, 0ull, 0ull, nullptr);
     if (wall) dE = INFINITY;   // beyond the container's wall
     if (ok && !wall) {
-        PT fene = (PT)0, tors = (PT)0;
-        bool near = false, tnear = false;
-        double part = (double)local_delta<32, PT>(d, P, M, s, g, sizeof(PT) == 4 ? &fene : nullptr, &near,
-                                                  sizeof(PT) == 4 ? &tors : nullptr, &tnear);
+        double part;
         if constexpr (sizeof(PT) == 4) {
+            float fene = 0.0f, tors = 0.0f;
+            bool near = false, tnear = false;
+            part = (double)local_delta32<32>(d, P, M, s, g, &fene, &near, &tors, &tnear);
             // a FENE bond near its divergence or a dihedral near degenerate: the exact
             // positions give that kind of term's change
             const bool fx = __ballot_sync(g.mask, near), tx = __ballot_sync(g.mask, tnear);
@@ -91,7 +91,7 @@ delta_kernel(const SysDesc d, int B, const double* __restrict__ xyz, const phast
                                        : pair_delta32<32, 3, false>(d, M, P.chain, s, g);
             part += (double)q.hi + (double)q.lo;
         } else {
-            part += pair_delta<32, PT, 4>(d, M, P.chain, s, g);
+            part = local_delta64<32>(d, P, M, s, g) + pair_delta64<32>(d, M, P.chain, s, g);
         }
         dE = g.sum(part);
     }

@@ -955,14 +955,14 @@ __device__ __noinline__ PT bond_item(const SysDesc& d, bool fene, P4<PT> a, P4<P
     return -f.kin() * lj_pair<PT>(a.x - b.x, a.y - b.y, a.z - b.z, (PT)0, (PT)0, f.C(2 * d.seq[l] + d.seq[l + 1]));
 }
 
-// fene (FP32): the FENE terms go to *fene rather than into the returned part,
-// and *near is set where one of them lies in the band of fene_w.  tors (FP32):
-// likewise the torsion terms go to *tors, and *tnear is set where a dihedral
-// lies in the band of torsion_w.
-template <int TPW, typename PT, bool GEOM = true>
-__device__ PT local_delta(const SysDesc& d, const Proposal& P, const MoveSet& M, const Slot<PT>& s,
-                              const Group<TPW>& g, PT* fene = nullptr, bool* near = nullptr, PT* tors = nullptr,
-                              bool* tnear = nullptr) {
+// FP32 local terms.  fene: the FENE terms go to *fene rather than into the returned part,
+// and *near is set where one of them lies in the band of fene_w.  tors: likewise the
+// torsion terms go to *tors, and *tnear is set where a dihedral lies in the band of
+// torsion_w.
+template <int TPW, bool GEOM = true>
+__device__ float local_delta32(const SysDesc& d, const Proposal& P, const MoveSet& M, const Slot<float>& s,
+                               const Group<TPW>& g, float* fene, bool* near, float* tors, bool* tnear) {
+    using PT = float;
     int vb0, nb, jt0, nt, fb0, nf;
     local_window(d, P.type, P.chain, P.index, &vb0, &nb, &jt0, &nt, &fb0, &nf);
     const int o = d.chain_off[P.chain];
@@ -975,15 +975,11 @@ __device__ PT local_delta(const SysDesc& d, const Proposal& P, const MoveSet& M,
         const int k = it >> 1;
         auto pos = [&](int j) -> P4<PT> {
             if (after && j >= M.lo && j <= M.hi) {
-                if constexpr (sizeof(PT) == 4) {
-                    const float4* mv = reinterpret_cast<const float4*>(s.newr) + 2 * rec_slot(d, M, j);
-                    const float4 a = mv[0], b = mv[1];
-                    P4<PT> w;
-                    w.x = a.y; w.y = a.w; w.z = b.y; w.tag = __float_as_int(b.z);
-                    return w;
-                } else {
-                    return s.newr[j - M.lo];
-                }
+                const float4* mv = reinterpret_cast<const float4*>(s.newr) + 2 * rec_slot(d, M, j);
+                const float4 a = mv[0], b = mv[1];
+                P4<PT> w;
+                w.x = a.y; w.y = a.w; w.z = b.y; w.tag = __float_as_int(b.z);
+                return w;
             }
             return s.r[j];
         };
@@ -991,12 +987,9 @@ __device__ PT local_delta(const SysDesc& d, const Proposal& P, const MoveSet& M,
         PT term;
         if (k < nb) term = f.kbend() * bend_w<PT>(pos, o, vb0 + k);
         else if (k < nb + nt) {
-            if (sizeof(PT) == 4 && tors) {
-                const PT v = -f.ktors() * torsion_w<PT>(pos, o, jt0 + (k - nb), tnear, GEOM);
-                *tors += after ? v : -v;
-                continue;
-            }
-            term = -f.ktors() * torsion_w<PT>(pos, o, jt0 + (k - nb));
+            const PT v = -f.ktors() * torsion_w<PT>(pos, o, jt0 + (k - nb), tnear, GEOM);
+            *tors += after ? v : -v;
+            continue;
         } else {   // a FENE bond or the bond move's pair: out of line (most workloads have neither)
             const bool is_fene = k < nb + nt + nf;
             const int l = o + (is_fene ? fb0 + (k - nb - nt) : P.index);   // the bond's first monomer
@@ -1164,65 +1157,97 @@ __device__ DF pair_delta32(const SysDesc& d, const MoveSet& M, int mchain, const
     return sum;
 }
 
-// This lane's share of the Lennard-Jones change in the working precision
-// (FP64 mode): unmoved partners t = lane, lane + TPW, ... (skipping the moved
-// range), R of them in registers at a time, each swept against every moved
-// monomer before and after the move, with the nearest-integer minimum image
-// between chains.
-template <int TPW, typename PT, int R>
-__device__ PT pair_delta(const SysDesc& d, const MoveSet& M, int mchain, const Slot<PT>& s,
-                         const Group<TPW>& g) {
-    const int m = M.hi - M.lo + 1;
-    const int U = d.N - m;
-    const int nc = d.n_chains;
-    const FF<PT> f{d};
-    const PT L = f.L(), iL = f.iL();
-    const PT kin = f.kin(), kout = f.kout();
-    const PT far = (PT)1.0e4;
-    PT part = (PT)0;
-    for (int t0 = g.lane; t0 < U; t0 += TPW * R) {
-        PT qx[R], qy[R], qz[R], Lj[R], iLj[R], C0[R], C1[R], kap[R], acc[R];
-#pragma unroll
-        for (int u = 0; u < R; ++u) {
-            const int t = t0 + u * TPW;
-            qx[u] = qy[u] = qz[u] = far;
-            Lj[u] = iLj[u] = C0[u] = C1[u] = kap[u] = (PT)0;
-            acc[u] = (PT)0;
-            if (t < U) {
-                const int j = t < M.lo ? t : t + m;
-                const P4<PT> p = s.r[j];
-                const int cj = p.tag >> 1, tj = p.tag & 1;
-                const bool ex = (j == M.ex0) | (j == M.ex1) | (j == M.ex2);
-                if (!ex) {
-                    if (cj == mchain) {
-                        qx[u] = p.x; qy[u] = p.y; qz[u] = p.z;
-                        kap[u] = kin;
-                    } else {
-                        const P4<PT> sh = s.D[mchain * nc + cj];
-                        qx[u] = p.x - sh.x; qy[u] = p.y - sh.y; qz[u] = p.z - sh.z;
-                        Lj[u] = L; iLj[u] = iL;
-                        kap[u] = kout;
-                    }
-                    C0[u] = f.C(tj);
-                    C1[u] = f.C(2 + tj);
-                }
-            }
+// This lane's share of the Lennard-Jones change in FP64: the evaluations (pair of a moved
+// and an unmoved monomer, before or after) as one flat list dealt to the lanes in turn.
+// An FP64 instruction holds the SMSP's FP64 pipe for 64 cycles however many lanes take
+// part, so what counts is the number of rounds: of a 13-mer's pivot (46 evaluations on
+// average) a full warp makes two, where four register partners a lane made twelve rounds
+// of mostly empty lanes.  13 FP64 instructions an evaluation, 16 with an image (26 with
+// rint images and a division).  Together with local_delta64 and the FP32 estimates of the
+// bin and of the exponential: a sweep of eight 13-mers takes 125 us, 417 us before.  The partners left out (move_set) are next to the moved
+// range, so the partners are the monomers outside one block.
+template <int TPW>
+__device__ double pair_delta64(const SysDesc& d, const MoveSet& M, int mchain, const Slot<double>& s,
+                               const Group<TPW>& g) {
+    int lo = M.lo, hi = M.hi;
+    if (M.ex1 >= 0 || (M.ex0 >= 0 && M.ex0 < M.lo)) --lo;
+    if (M.ex2 >= 0 || M.ex0 > M.hi) ++hi;
+    const int blk = hi - lo + 1, U = d.N - blk;
+    const int pairs = (M.hi - M.lo + 1) * U;
+    if (pairs == 0) return 0.0;
+    const bool after = g.lane & 1;   // TPW is even: a lane keeps to the old or the new positions
+    const P4<double>* moved = after ? s.newr : s.r + M.lo;
+    const int dq = (TPW / 2) / U, dt = (TPW / 2) % U;
+    int q = (g.lane >> 1) / U, t = (g.lane >> 1) % U;
+    double acc_in = 0.0, acc_out = 0.0;
+    for (int p = g.lane >> 1; p < pairs; p += TPW / 2) {
+        const P4<double> a = moved[q], b = s.r[t < lo ? t : t + blk];
+        const bool inter = (b.tag >> 1) != mchain;
+        double dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
+        if (inter) {
+            dx = mimage64_short(d, dx);
+            dy = mimage64_short(d, dy);
+            dz = mimage64_short(d, dz);
         }
-#pragma unroll 2
-        for (int i = 0; i < m; ++i) {
-            const P4<PT> a = s.r[M.lo + i];
-            const P4<PT> b = s.newr[i];
-            const bool ib = a.tag & 1;
-#pragma unroll
-            for (int u = 0; u < R; ++u) {
-                const PT C = ib ? C1[u] : C0[u];
-                const PT e0 = lj_pair<PT>(a.x - qx[u], a.y - qy[u], a.z - qz[u], Lj[u], iLj[u], C);
-                const PT e1 = lj_pair<PT>(b.x - qx[u], b.y - qy[u], b.z - qz[u], Lj[u], iLj[u], C);
-                acc[u] += e1 - e0;
+        const double ir2 = rcp64(dx * dx + dy * dy + dz * dz);
+        const double ir6 = ir2 * ir2 * ir2;
+        const double w = flip_sign(ir6 - d.C[2 * (a.tag & 1) + (b.tag & 1)], !after);
+        const double acc = __fma_rn(ir6, w, inter ? acc_out : acc_in);
+        acc_in = inter ? acc_in : acc;
+        acc_out = inter ? acc : acc_out;
+        q += dq;
+        t += dt;
+        if (t >= U) { t -= U; ++q; }
+    }
+    return d.k_lj_intra * acc_in + d.k_lj_inter * acc_out;
+}
+
+// This lane's share of the bending, torsion and FENE change in FP64.  A bend is the cosine
+// between two bonds, a dihedral the cosine between two normals: once a lane has its two
+// vectors both take the same instructions.
+template <int TPW, bool GEOM = true>
+__device__ double local_delta64(const SysDesc& d, const Proposal& P, const MoveSet& M, const Slot<double>& s,
+                                const Group<TPW>& g) {
+    int vb0, nb, jt0, nt, fb0, nf;
+    local_window(d, P.type, P.chain, P.index, &vb0, &nb, &jt0, &nt, &fb0, &nf);
+    const int o = d.chain_off[P.chain];
+    if (d.k_tors == 0.0) nt = 0;
+    if (!GEOM) nf = 0;
+    const int nc = GEOM && P.type == PHAST_BOND;   // the stretched bond's pair, counted by the pair loop, taken back
+    double part = 0.0;
+    for (int it = g.lane; it < 2 * (nb + nt + nf + nc); it += TPW) {
+        const bool after = it & 1;
+        const int k = it >> 1;
+        auto pos = [&](int j) -> P4<double> {
+            return (after && j >= M.lo && j <= M.hi) ? s.newr[j - M.lo] : s.r[j];
+        };
+        double term;
+        if (k < nb + nt) {
+            const bool tors = k >= nb;
+            const int j = o + (tors ? jt0 + (k - nb) : vb0 + k - 1);
+            const P4<double> x0 = pos(j), x1 = pos(j + 1), x2 = pos(j + 2);
+            double ux = x1.x - x0.x, uy = x1.y - x0.y, uz = x1.z - x0.z;
+            double wx = x2.x - x1.x, wy = x2.y - x1.y, wz = x2.z - x1.z;
+            if (tors) {
+                const P4<double> x3 = pos(j + 3);
+                const double cx = x3.x - x2.x, cy = x3.y - x2.y, cz = x3.z - x2.z;
+                const double nx = uy * wz - uz * wy, ny = uz * wx - ux * wz, nz = ux * wy - uy * wx;
+                const double mx = wy * cz - wz * cy, my = wz * cx - wx * cz, mz = wx * cy - wy * cx;
+                ux = nx; uy = ny; uz = nz;
+                wx = mx; wy = my; wz = mz;
             }
+            const double uw = ux * wx + uy * wy + uz * wz;
+            const double p = (ux * ux + uy * uy + uz * uz) * (wx * wx + wy * wy + wz * wz);
+            const double c = uw * rsqrt64(p);
+            // p >= 0: its bit pattern orders as its value
+            const bool degenerate = tors && __double_as_longlong(p) < __double_as_longlong(1e-20);
+            term = tors ? (degenerate ? 0.0 : -d.k_tors * c) : d.k_bend * (1.0 - c);
+        } else {
+            const bool is_fene = k < nb + nt + nf;
+            const int l = o + (is_fene ? fb0 + (k - nb - nt) : P.index);   // the bond's first monomer
+            term = bond_item<double>(d, is_fene, pos(l), pos(l + 1), l);
         }
-#pragma unroll
-        for (int u = 0; u < R; ++u) part += kap[u] * acc[u];
+        part += flip_sign(term, !after);
     }
     return part;
 }
@@ -1243,20 +1268,16 @@ __device__ __forceinline__ int bin_after(const SysDesc& d, double E, float erel,
 }
 
 // The acceptance test for dlnW < 0: u < exp(dlnW), decided exactly as in
-// FP64.  FP32 mode settles it with an FP32 exponential and the top 24 bits of
-// u whenever they are further apart than their error bounds (|u - u24| <=
+// FP64.  An FP32 exponential and the top 24 bits of u settle it whenever they are further apart than their error bounds (|u - u24| <=
 // 2^-24; expf within 2 ulp; the FP32 rounding of dlnW adds |dlnW| 2^-24
 // relative), and falls back to FP64 in the rare near-tie.
-template <typename PT>
 __device__ __forceinline__ bool accept_below(double dl, const Proposal& P) {
-    if constexpr (sizeof(PT) == 4) {
-        const float dlf = (float)dl;
-        const float e = expf(dlf);
-        const float u24 = ((float)(P.uz >> 8) + 0.5f) * 5.9604644775390625e-8f;
-        const float rel = 5e-7f + fabsf(dlf) * 1.2e-7f;
-        if (u24 + 6e-8f < e * (1.0f - rel)) return true;
-        if (u24 - 6e-8f > e * (1.0f + rel)) return false;
-    }
+    const float dlf = (float)dl;
+    const float e = expf(dlf);
+    const float u24 = ((float)(P.uz >> 8) + 0.5f) * 5.9604644775390625e-8f;
+    const float rel = 5e-7f + fabsf(dlf) * 1.2e-7f;
+    if (u24 + 6e-8f < e * (1.0f - rel)) return true;
+    if (u24 - 6e-8f > e * (1.0f + rel)) return false;
     return u52(P.uz, P.uw) < exp(dl);
 }
 

@@ -397,7 +397,7 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
             lnw_new = __ldg(lnW + b_new);
             const double dl = lnw_new - lnw_here;
             if (GEOM && P.type == PHAST_BOND) acc = accept_stretch(dl, jac, P);
-            else acc = (dl >= 0.0) || accept_below<PT>(dl, P);
+            else acc = (dl >= 0.0) || accept_below(dl, P);
         }
         if (acc) {
             E = E + (sizeof(PT) == 4 ? (double)dE32.hi + (double)dE32.lo : dE64);

@@ -200,8 +200,8 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
                                       : pair_delta32<TPW, 3, false>(sd, M, P.chain, slot, g);
                 float fene = 0.0f, tors = 0.0f;
                 bool near = false, tnear = false;
-                part = df_add(part, DF{local_delta<TPW, PT, GEOM>(sd, P, M, slot, g, GEOM ? &fene : nullptr,
-                                                                  &near, &tors, &tnear), 0.0f});
+                part = df_add(part, DF{local_delta32<TPW, GEOM>(sd, P, M, slot, g, GEOM ? &fene : nullptr, &near,
+                                                                &tors, &tnear), 0.0f});
                 if constexpr (GEOM) {
                     // a FENE bond near its divergence or a dihedral near degenerate: the
                     // exact positions give that kind of term's change
@@ -226,19 +226,19 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
             dE32 = group_sum_df<TPW>(part, g);
         } else {
             double part = 0.0;
-            if (eval) part = local_delta<TPW, PT, GEOM>(sd, P, M, slot, g) + pair_delta<TPW, PT, 4>(sd, M, P.chain, slot, g);
+            if (eval) part = local_delta64<TPW, GEOM>(sd, P, M, slot, g) + pair_delta64<TPW>(sd, M, P.chain, slot, g);
             dE64 = g.sum(part);
         }
         const bool finite = eval && (sizeof(PT) == 4 ? (isfinite(dE32.hi) && isfinite(dE32.lo)) : isfinite(dE64));
         int b_new = -1;
-        if (finite) b_new = sizeof(PT) == 4 ? bin_after(sd, E, erel, dE32) : bin_of(sd, E + dE64);
+        if (finite) b_new = sizeof(PT) == 4 ? bin_after(sd, E, erel, dE32) : bin_of_short(sd, E + dE64);
         const double lnw_new = __ldg(lnW + (b_new >= 0 ? b_new : bin));
         blk = stream_block<OUT>(seed, t + 1, (uint32_t)g.lane);   // next move's block, while the load is in flight
         bool acc = false;
         if (b_new >= 0) {
             const double dl = lnw_new - lnw_here;
             if (GEOM && P.type == PHAST_BOND) acc = accept_stretch(dl, jac, P);
-            else acc = (dl >= 0.0) || accept_below<PT>(dl, P);
+            else acc = (dl >= 0.0) || accept_below(dl, P);
         }
         if (acc) {
             E = E + (sizeof(PT) == 4 ? (double)dE32.hi + (double)dE32.lo : dE64);
