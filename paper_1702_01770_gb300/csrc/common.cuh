@@ -52,6 +52,7 @@ struct SysDesc {
     float amax32[PHAST_N_MOVES], pad3[2];
     float fene_r0_32, fene_iR32, fene_kR2_32, pad4;
     float C_F32[4];
+    double inv_len[PHAST_MAX_CHAINS];   // 1 / chain length, correctly rounded
     int32_t chain_off[PHAST_MAX_CHAINS + 1];
     int32_t pad1[3];
     uint8_t seq[PHAST_MAX_MONOMERS];
@@ -131,10 +132,46 @@ __device__ __forceinline__ double u52(uint32_t a, uint32_t b) {
 __device__ __forceinline__ uint64_t u52_bits(uint32_t a, uint32_t b) {
     return ((uint64_t)(a >> 6) << 26) | (uint64_t)(b >> 6);
 }
-// 2u - 1 = (2n + 1 - 2^52) 2^-52, exact.
+// 2u - 1 = (2n + 1 - 2^52) 2^-52, exact: the odd integer's bits put in place (a conversion
+// or a product in FP64 would hold the FP64 pipe for 64 to 95 cycles each).
 __device__ __forceinline__ double sym_unit(uint32_t a, uint32_t b) {
-    int64_t k = (int64_t)(2 * u52_bits(a, b) + 1) - (int64_t)(1ull << 52);
-    return xmul((double)k, 2.220446049250313080847263336181640625e-16);
+    const int64_t k = (int64_t)(2 * u52_bits(a, b) + 1) - (int64_t)(1ull << 52);
+    const uint64_t m = (uint64_t)(k < 0 ? -k : k);   // odd, below 2^52
+    const int lz = __clzll((long long)m);
+    const uint64_t bits = ((uint64_t)(1033 - lz) << 52) + (m << (lz - 11));   // the leading one adds 1 to the exponent
+    return __longlong_as_double((long long)(bits | (k < 0 ? 1ull << 63 : 0ull)));
+}
+
+// FP32 -> FP64 and FP64 -> FP32 (round to nearest even), the same values as the
+// conversions, from the bits: about ten integer instructions instead of 92 cycles of the
+// FP64 pipe.  Zero, subnormal, infinite and NaN values and results take the conversion.
+__device__ __forceinline__ double f32_to_f64(float f) {
+    const int b = __float_as_int(f), a = b & 0x7fffffff;
+    if ((unsigned)(a - 0x00800000) >= 0x7f000000u) return (double)f;
+    return __hiloint2double((b & 0x80000000) | ((a >> 3) + 0x38000000), b << 29);
+}
+__device__ __forceinline__ float f64_to_f32(double x) {
+    const int hi = __double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    const unsigned a = (unsigned)hi & 0x7fffffffu;
+    if (a - 0x38100000u >= 0x0fd00000u) return (float)x;   // below 2^-126 or above 2^127
+    unsigned r = ((a - 0x38000000u) << 3) | (lo >> 29);
+    const unsigned rest = lo << 3;   // the dropped bits, the half at the top
+    r += (rest > 0x80000000u) || (rest == 0x80000000u && (r & 1u));
+    return __int_as_float((int)(r | ((unsigned)hi & 0x80000000u)));
+}
+// A small count (1 .. 2^20) in FP64, from its bits.
+__device__ __forceinline__ double count_to_f64(int n) {
+    const int lz = __clz(n);
+    return __hiloint2double(((1053 - lz) << 20) + (int)(((unsigned)n << lz) >> 11), 0);
+}
+// x / n rounded correctly, for a chain length n with rn = 1/n correctly rounded: the
+// quotient x rn and one correction by its exact residual (Markstein's division).  The
+// residual x - n q is exact, and x / n keeps at least 2^-10 of an ulp from the midpoints of
+// the FP64 numbers for n < 2^10, far more than the correction's own rounding.
+__device__ __forceinline__ double div_count(double x, double n, double rn) {
+    const double q = __dmul_rn(x, rn);
+    return __fma_rn(__fma_rn(-q, n, x), rn, q);
 }
 
 // sin and cos of |a| <= 1 by their Taylor series, Horner in a^2 with separately
@@ -196,8 +233,10 @@ __device__ __forceinline__ bool marsaglia_in_disc(uint4 r, double* v1, double* v
     return *s < 1.0 && *s > 0.0;
 }
 __device__ __forceinline__ double3 marsaglia_axis(double v1, double v2, double s) {
-    double q = xsqrt(xsub(1.0, s));
-    return make_double3(xmul(xmul(2.0, v1), q), xmul(xmul(2.0, v2), q), xsub(1.0, xmul(2.0, s)));
+    // (2 v) q = v (2 q) and 1 - 2 s in one rounding each; 2 q by its exponent (0 < q < 1)
+    const double q = xsqrt(xsub(1.0, s));
+    const double q2 = __hiloint2double(__double2hiint(q) + 0x00100000, __double2loint(q));
+    return make_double3(xmul(v1, q2), xmul(v2, q2), xfma(-2.0, s, 1.0));
 }
 __device__ __forceinline__ bool marsaglia_try(uint4 r, double3* axis) {
     double v1, v2, s;
@@ -306,7 +345,7 @@ __device__ __forceinline__ int bin_of(const SysDesc& d, double E) {
 // bin_of, the division by the bin width taken only where an FP32 estimate of the
 // quotient (error under 2e-7 of it) lies within its error of a bin edge.
 __device__ __forceinline__ int bin_of_short(const SysDesc& d, double E) {
-    const float x = (float)xsub(E, d.e_min) * d.iw32;
+    const float x = f64_to_f32(xsub(E, d.e_min)) * d.iw32;
     const float fl = floorf(x), fr = x - fl, mg = 4e-7f * fabsf(x) + 1e-6f;
     if (fr > mg && fr < 1.0f - mg) return (fl < 0.0f || fl >= (float)d.n_bins) ? -1 : (int)fl;
     return bin_of(d, E);
@@ -384,9 +423,10 @@ __device__ __forceinline__ double3 ld3(const double* p) { return make_double3(p[
 // or a step through zero length.  *jac: the move's Hastings factor
 // ((r + delta) / r)^2, the Jacobian determinant of the radial map of the bond
 // vector (bead coordinates are the sampled measure).
-__device__ __forceinline__ bool bond_step(const double* x64, int o, int n, int l, double delta, double3* step,
+template <class Pos>
+__device__ __forceinline__ bool bond_step(const Pos& pos, int o, int n, int l, double delta, double3* step,
                                           double* jac) {
-    const double3 a = ld3(x64 + 3 * (o + l)), b = ld3(x64 + 3 * (o + l + 1));
+    const double3 a = pos(o + l), b = pos(o + l + 1);
     const double bx = xsub(b.x, a.x), by = xsub(b.y, a.y), bz = xsub(b.z, a.z);
     const double len = xsqrt(xadd(xadd(xmul(bx, bx), xmul(by, by)), xmul(bz, bz)));
     if (!(len > 1e-12) || !(xadd(len, delta) > 0.0)) return false;

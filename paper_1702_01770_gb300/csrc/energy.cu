@@ -97,7 +97,7 @@ delta_kernel(const SysDesc d, int B, const double* __restrict__ xyz, const phast
     }
     if (g.lane == 0) dE_out[b] = dE;
     if (xyz_new) {
-        if (sizeof(PT) == 4 && valid) prepare_exact<32, PT>(d, x64, P, P.axis, s, g);
+        if (sizeof(PT) == 4 && valid) prepare_exact<32, PT>(d, [&](int j) { return ld3(x64 + 3 * j); }, P, P.axis, s, g);
         double* out = xyz_new + (size_t)b * d.N * 3;
         for (int j = g.lane; j < d.N; j += 32) {
             double3 y = ld3(x64 + 3 * j);

@@ -45,7 +45,7 @@ struct LaneSlot {
 
 // Full FP64 energy (Eq. 2 per chain + the inter-chain term of Eq. 3, torsion,
 // FENE bonds and the container) of one walker by one thread.
-__device__ double lane_energy64(const SysDesc& d, const double* x64) {
+static __device__ double lane_energy64(const SysDesc& d, const double* x64) {
     auto pos = [&](int j) -> double3 { return ld3(x64 + 3 * j); };
     double e = 0.0;
     bool out = false;
@@ -145,7 +145,7 @@ __device__ __forceinline__ bool lane_geometry(const SysDesc& d, const double* x6
         G->step = P.disp;
         return true;
     }
-    if (GEOM && P.type == PHAST_BOND) return bond_step(x64, o, n, P.index, P.angle, &G->step, jac);
+    if (GEOM && P.type == PHAST_BOND) return bond_step([&](int j) { return ld3(x64 + 3 * j); }, o, n, P.index, P.angle, &G->step, jac);
     double3 axis = P.axis;
     if (P.type == PHAST_PIVOT) {
         G->c = ld3(x64 + 3 * (o + P.index));
