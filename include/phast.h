@@ -310,7 +310,7 @@ int phast_energy_grad_params(const phast_system* sys, const phast_ff* ff, int32_
  *   dcV_T = [2 <(E-<E>)(D-<D>)> - beta <(E-<E>)^2 (D-<D>)>] / (N T^2),
  * from d<O>/dlambda = <dO/dlambda> - beta Cov(O, D) for O = E and E^2.
  * All arrays on the device, FP64: E, D, lnW [n]; T, E_T, cV_T, dE_T, dcV_T [n_T].
- * One CTA per temperature.  PHAST_EINVAL for bad arguments. */
+ * One cluster of CTAs per temperature.  PHAST_EINVAL for bad arguments. */
 int phast_reweight_sensitivity(int64_t n, const double* E, const double* D, const double* lnW,
                                int32_t n_monomers, int32_t n_T, const double* T, double* E_T,
                                double* cV_T, double* dE_T, double* dcV_T, void* stream);

@@ -62,12 +62,18 @@ struct SysDesc {
 };
 static_assert(sizeof(SysDesc) % 16 == 0, "SysDesc must be 16-byte sized for vector copies");
 
-// Validates the ABI structs and fills a descriptor (offsets left at 0).
-// Berg step on stream st (weights.cu); set_attr: set the kernel's shared-memory
-// limit first (not allowed while a stream is being captured).
-int phast_launch_berg(int32_t K, double bin_width, const uint64_t* hist, int32_t n_blocks, double* lnW,
-                      double* g_acc, double* beta_out, double* flat_out, cudaStream_t st, bool set_attr);
+// One step of Berg's recursion for up to PHAST_MAX_SYSTEMS types in one launch on stream st
+// (weights.cu); the fields as phast_weight_update's arguments.
+struct BergJob {
+    int32_t K, n_blocks;
+    double w;
+    const unsigned long long* hist;
+    double *lnW, *g_acc, *beta_out, *flat_out;
+};
+struct BergJobs { BergJob job[PHAST_MAX_SYSTEMS]; };
+int phast_launch_berg(const BergJobs& jobs, int n_jobs, cudaStream_t st);
 
+// Validates the ABI structs and fills a descriptor (offsets left at 0).
 int phast_build_desc(const phast_system* sys, const phast_ff* ff, const phast_muca_params* mp,
                      SysDesc* d, const char* what);
 
@@ -494,6 +500,31 @@ __device__ __forceinline__ double rsqrt64(double x) {
 }
 __device__ __forceinline__ double flip_sign(double x, bool flip) {
     return __hiloint2double(__double2hiint(x) ^ (flip ? (int)0x80000000 : 0), __double2loint(x));
+}
+
+// Warp sums of N values per lane: at each step a lane passes half of its values on and adds
+// up the other half, so N values take about N additions (20 for 18) instead of 5 N, which
+// counts where an addition holds the FP64 pipe for 64 cycles.  first: index of the lane's
+// v[0], count: how many of its v are values.  Ends with the sum of value *first in v[0] where
+// *count is 1 (nothing where it is 0; some sums end on more than one lane).
+template <int N, int O = 16>
+__device__ __forceinline__ void warp_sums(double* v, int* first, int* count) {
+    if constexpr (N > 1) {
+        constexpr int half = (N + 1) / 2;
+        const bool upper = threadIdx.x & O;
+#pragma unroll
+        for (int j = 0; j < half; ++j) {
+            const double hi = half + j < N ? v[half + j] : 0.0;
+            const double got = __shfl_xor_sync(0xffffffffu, upper ? v[j] : hi, O);
+            v[j] = (upper ? hi : v[j]) + got;
+        }
+        if (upper) *first += half;
+        *count = upper ? max(*count - half, 0) : min(*count, half);
+        if constexpr (O > 1) warp_sums<half, O / 2>(v, first, count);
+    } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+        if constexpr (O > 1) warp_sums<1, O / 2>(v, first, count);
+    }
 }
 
 // Block-wide FP64 sum; every thread gets the result.  red: >= 32 doubles of shared.

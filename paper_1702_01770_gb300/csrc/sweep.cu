@@ -902,14 +902,12 @@ extern "C" int phast_ctx_capture_iteration(phast_ctx* c, int64_t n_sweeps, doubl
     if (n_sweeps < 1) return phast_set_error(PHAST_EINVAL, "phast_ctx_capture_iteration: n_sweeps < 1");
     if (n_jk < 1) return phast_set_error(PHAST_EINVAL, "phast_ctx_capture_iteration: n_jk < 1");
     const bool fp32 = c->desc[0].pair_precision == 32;
-    int max_bins = 1;
     size_t hs_bytes = 0;
     for (int s = 0; s < c->n_sys; ++s) {
         if (n_jk > c->desc[s].n_walkers)
             return phast_set_error(PHAST_EINVAL, "phast_ctx_capture_iteration: n_jk %d > walkers of system %d", n_jk, s);
         if ((c->desc[s].pair_precision == 32) != fp32)
             return phast_set_error(PHAST_EINVAL, "phast_ctx_capture_iteration: system types mix pair precisions");
-        max_bins = std::max(max_bins, (int)c->desc[s].n_bins);
         hs_bytes += sizeof(uint64_t) * (size_t)n_jk * (size_t)c->desc[s].n_bins;
     }
     SweepArgs a;
@@ -917,20 +915,19 @@ extern "C" int phast_ctx_capture_iteration(phast_ctx* c, int64_t n_sweeps, doubl
     BatchedLaunch L;
     int rc = prepare_batched(c, a, c->tpw, c->wpc, fp32, &L);
     if (rc != PHAST_OK) return rc;
-    // the Berg kernel's shared-memory limit is set outside the capture
-    rc = phast_launch_berg(max_bins, 1.0, nullptr, 1, nullptr, nullptr, nullptr, nullptr, nullptr, true);
-    if (rc != PHAST_OK) return rc;
+    BergJobs jobs = {};
+    for (int s = 0; s < c->n_sys; ++s) {
+        const SysDesc& d = c->desc[s];
+        jobs.job[s] = BergJob{d.n_bins, n_jk, d.bin_width, reinterpret_cast<const unsigned long long*>(hist_sum + a.hs_off[s]),
+                              lnW + d.lnw_off, g_acc + d.lnw_off, nullptr, flat_out ? flat_out + 4 * s : nullptr};
+    }
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return phast_set_error(PHAST_ECUDA, "phast_ctx_capture_iteration: %s", cudaGetErrorString(e));
     rc = PHAST_OK;
     if (cudaMemsetAsync(hist_sum, 0, hs_bytes, st) != cudaSuccess) rc = PHAST_ECUDA;
     if (rc == PHAST_OK) rc = enqueue_batched(c, L, st);
-    for (int s = 0; s < c->n_sys && rc == PHAST_OK; ++s) {
-        const SysDesc& d = c->desc[s];
-        rc = phast_launch_berg(d.n_bins, d.bin_width, hist_sum + a.hs_off[s], n_jk, lnW + d.lnw_off, g_acc + d.lnw_off,
-                               nullptr, flat_out ? flat_out + 4 * s : nullptr, st, false);
-    }
+    if (rc == PHAST_OK) rc = phast_launch_berg(jobs, c->n_sys, st);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(st, &graph);
     if (rc != PHAST_OK || e != cudaSuccess) {
