@@ -299,6 +299,25 @@ int phast_energy_grad_params(const phast_system* sys, const phast_ff* ff, int32_
                              int32_t pair_precision, const double* params, double* E_out,
                              double* grad_xyz, double* grad_ff, void* stream);
 
+/* The forward and the backward pass of a training step, with FP32 pair terms
+ * (phast_energy_grad's pair_precision 32) and without the passes over the
+ * batch around it.  xyz: dev [B][N][3], FP32 (xyz_bits 32) or FP64 (64);
+ * params: as for phast_energy_grad_params, FP32 or FP64 by params_bits, or NULL
+ * for ff's values.
+ *  forward: E_out dev FP64 [B].
+ *  backward: grad_E dev FP64 [B] (dloss/dE); grad_xyz in the type of xyz,
+ * dloss/dx = grad_E dE/dx, or NULL; grad_params dev [5] in the type of params,
+ * dloss/dparams summed over the batch in FP64, or NULL; workspace dev [PHAST_VJP_DOUBLES] FP64,
+ * needed with grad_params.  Nothing is kept from the forward pass (it is
+ * recomputed).  PHAST_EINVAL for bad arguments. */
+#define PHAST_VJP_DOUBLES 12160
+int phast_energy_forward32(const phast_system* sys, const phast_ff* ff, int32_t B, const void* xyz,
+                           int32_t xyz_bits, const void* params, int32_t params_bits, double* E_out,
+                           void* stream);
+int phast_energy_backward32(const phast_system* sys, const phast_ff* ff, int32_t B, const void* xyz,
+                            int32_t xyz_bits, const void* params, int32_t params_bits, const double* grad_E,
+                            void* grad_xyz, void* grad_params, double* workspace, void* stream);
+
 /* Canonical averages from multicanonical samples (Sec. 2.2 reweighting) and
  * their derivatives in a force-field parameter lambda.  Sample q (of n) has
  * energy E[q], D[q] = dE/dlambda (e.g. a column of grad_ff) and was drawn with

@@ -30,7 +30,8 @@ SYMBOLS = ["phast_energy", "phast_delta_energy", "phast_ctx_create", "phast_ctx_
            "phast_version", "phast_ctx_capture_iteration", "phast_graph_launch",
            "phast_graph_destroy", "phast_energy_grad",
            "phast_reweight_sensitivity", "phast_maxwell", "phast_micro_binned_workspace_size",
-           "phast_micro_analysis_binned", "phast_ctx_set_hist_flush", "phast_energy_grad_params"]
+           "phast_micro_analysis_binned", "phast_ctx_set_hist_flush", "phast_energy_grad_params",
+           "phast_energy_forward32", "phast_energy_backward32"]
 
 
 class PhastError(RuntimeError):
@@ -109,6 +110,8 @@ def lib():
         L.phast_maxwell.argtypes = [i32, dbl, dbl, vp, vp, i32, i32, i32, dbl, dbl, dbl, vp, vp, vp, vp]
         L.phast_energy_grad.argtypes = [P(_System), P(_FF), i32, vp, i32, vp, vp, vp, vp]
         L.phast_energy_grad_params.argtypes = [P(_System), P(_FF), i32, vp, i32, vp, vp, vp, vp, vp]
+        L.phast_energy_forward32.argtypes = [P(_System), P(_FF), i32, vp, i32, vp, i32, vp, vp]
+        L.phast_energy_backward32.argtypes = [P(_System), P(_FF), i32, vp, i32, vp, i32, vp, vp, vp, vp, vp]
         L.phast_reweight_sensitivity.argtypes = [i64, vp, vp, vp, i32, i32, vp, vp, vp, vp, vp, vp]
         L.phast_ctx_capture_iteration.argtypes = [vp, i64, vp, i32, vp, vp, vp, P(vp), vp]
         L.phast_graph_launch.argtypes = [vp, vp]
@@ -227,29 +230,60 @@ def phast_energy_grad(system, xyz: torch.Tensor, pair_precision: int = 32, want_
     return E, gx, gf
 
 
+VJP_DOUBLES = 12160   # PHAST_VJP_DOUBLES
+_BITS = {torch.float32: 32, torch.float64: 64}
+
+
+def _device_params(params: torch.Tensor, xyz: torch.Tensor) -> torch.Tensor:
+    """The five parameters contiguous beside xyz, in FP32 or FP64 as they are (FP64 for other types)."""
+    assert params.numel() == 5
+    dtype = params.dtype if params.dtype in _BITS else torch.float64
+    return params.to(device=xyz.device, dtype=dtype).contiguous()
+
+
 class EnergyFunction(torch.autograd.Function):
     """E(xyz, params) for a batch of conformations of one system; params are the five
     force-field parameters (ff_params order).  The backward pass recomputes the forward
-    one in the same kernel (nothing is kept but the inputs)."""
+    one in the same kernel (nothing is kept but the inputs).  With FP32 pair terms, FP32 and
+    FP64 coordinates are read and their gradients written as they are (scaled by the incoming
+    gradient and, for the parameters, summed in the kernel)."""
 
     @staticmethod
     def forward(ctx, xyz, params, system, pair_precision):
         # the parameters stay where they are (no copy to the host, no synchronisation)
-        p = params.detach().to(device=xyz.device, dtype=torch.float64).contiguous()
-        E, _, _ = phast_energy_grad(system, xyz.detach().to(torch.float64), pair_precision, want_xyz=False,
-                                    want_ff=False, params=p)
         ctx.save_for_backward(xyz, params)
         ctx.system, ctx.pair_precision = system, pair_precision
-        return E
+        if pair_precision == 32 and xyz.dtype in _BITS:
+            x, p = xyz.contiguous(), _device_params(params, xyz)
+            ctx.structs = st = _Structs([system])
+            B = x.shape[0] if x.numel() else 0
+            E = torch.empty(B, dtype=torch.float64, device=x.device)
+            _check(lib().phast_energy_forward32(st.sys, st.ff, B, _ptr(x), _BITS[x.dtype], _ptr(p), _BITS[p.dtype],
+                                                _ptr(E), _stream(None)))
+            return E
+        p = params.detach().to(device=xyz.device, dtype=torch.float64).contiguous()
+        return phast_energy_grad(system, xyz.detach().to(torch.float64), pair_precision, want_xyz=False, want_ff=False,
+                                 params=p)[0]
 
     @staticmethod
     def backward(ctx, gE):
         xyz, params = ctx.saved_tensors
+        want_xyz, want_par = ctx.needs_input_grad[:2]
+        if ctx.pair_precision == 32 and xyz.dtype in _BITS:
+            x, p, st = xyz.contiguous(), _device_params(params, xyz), ctx.structs
+            gE = gE.to(torch.float64).contiguous()
+            B = x.shape[0] if x.numel() else 0
+            g_xyz = torch.empty_like(x) if want_xyz else None
+            g_par = torch.empty_like(p) if want_par else None
+            ws = torch.empty(VJP_DOUBLES, dtype=torch.float64, device=x.device) if want_par else None
+            _check(lib().phast_energy_backward32(st.sys, st.ff, B, _ptr(x), _BITS[x.dtype], _ptr(p), _BITS[p.dtype],
+                                                 _ptr(gE), _ptr(g_xyz), _ptr(g_par), _ptr(ws), _stream(None)))
+            return g_xyz, g_par.to(params.device, params.dtype) if want_par else None, None, None
         p = params.detach().to(device=xyz.device, dtype=torch.float64).contiguous()
         _, gx, gf = phast_energy_grad(ctx.system, xyz.detach().to(torch.float64), ctx.pair_precision, params=p)
         gE = gE.to(torch.float64)
-        g_xyz = (gE.view(-1, 1, 1) * gx).to(xyz.dtype) if ctx.needs_input_grad[0] else None
-        g_par = (gE.view(-1, 1) * gf).sum(0).to(params.device, params.dtype) if ctx.needs_input_grad[1] else None
+        g_xyz = (gE.view(-1, 1, 1) * gx).to(xyz.dtype) if want_xyz else None
+        g_par = (gE.view(-1, 1) * gf).sum(0).to(params.device, params.dtype) if want_par else None
         return g_xyz, g_par, None, None
 
 
