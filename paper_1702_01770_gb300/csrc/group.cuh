@@ -1407,6 +1407,41 @@ __device__ __forceinline__ bool accept_stretch(double dl, double J, const Propos
     return u52(P.uz, P.uw) < J * exp(dl);
 }
 
+// Bending, torsion and FENE energies of a configuration in FP64, this lane's share, by one of
+// `n_warps` warps (number `warp`).  The warp holds 32 consecutive monomers, one a lane;
+// bonds, their squares, the normals of neighbouring bonds and the normals' squares are each
+// formed once and passed down the lanes, so a monomer's bend and dihedral take 38 FP64
+// instructions (62 and two square roots and a division each from the positions).
+static __device__ double local_energy64_warp(const SysDesc& d, const double* x64, int lane, int warp, int n_warps) {
+    const unsigned full = 0xffffffffu;
+    double part = 0.0;
+    auto next = [&](double v) { return __shfl_down_sync(full, v, 1); };
+    for (int base = 29 * warp; base < d.N - 1; base += 29 * n_warps) {   // terms that begin at base .. base + 28
+        const int i = base + lane;
+        const double3 x = ld3(x64 + 3 * min(i, d.N - 1));
+        const int c = i < d.N ? d.chain_of[i] : -1;
+        const int c1 = i + 1 < d.N ? d.chain_of[i + 1] : -2, c2 = i + 2 < d.N ? d.chain_of[i + 2] : -2,
+                  c3 = i + 3 < d.N ? d.chain_of[i + 3] : -2;
+        const double bx = next(x.x) - x.x, by = next(x.y) - x.y, bz = next(x.z) - x.z;
+        const double bb = bx * bx + by * by + bz * bz;
+        const double ex = next(bx), ey = next(by), ez = next(bz), ee = next(bb);
+        const bool mine = lane < 29;
+        if (mine && c2 == c) part += d.k_bend * (1.0 - (bx * ex + by * ey + bz * ez) * rsqrt64(bb * ee));
+        if (d.k_tors != 0.0) {
+            const double nx = by * ez - bz * ey, ny = bz * ex - bx * ez, nz = bx * ey - by * ex;
+            const double nn = nx * nx + ny * ny + nz * nz;
+            const double mx = next(nx), my = next(ny), mz = next(nz), mm = next(nn);
+            const double p = nn * mm;
+            // p >= 0: its bit pattern orders as its value (NaN above: a bad configuration's term)
+            if (mine && c3 == c && __double_as_longlong(p) >= __double_as_longlong(1e-20))
+                part -= d.k_tors * ((nx * mx + ny * my + nz * mz) * rsqrt64(p));
+        }
+        if (d.k_fene != 0.0 && mine && c1 == c)
+            part += fene_term(d, [&](int j) { return ld3(x64 + 3 * j); }, i, 0);
+    }
+    return part;
+}
+
 // Full FP64 energy (Eq. 2 per chain + inter-chain term of Eq. 3) of the
 // walker at x64; every lane of the group receives the total.
 template <int TPW>
@@ -1443,25 +1478,18 @@ __device__ double full_energy64(const SysDesc& d, const double* x64, const Group
     return __any_sync(g.mask, out) ? INFINITY : E;
 }
 
-// Full energy with the Lennard-Jones pairs in the working precision (from the
-// working copy) and the local terms in FP64 (from x64).
-template <int TPW, typename PT>
-__device__ double full_energy_working(const SysDesc& d, const double* x64, const Slot<PT>& s, const Group<TPW>& g) {
-    double part = 0.0;
-    auto pos = [&](int j) -> double3 { return ld3(x64 + 3 * j); };
-    for (int c = 0; c < d.n_chains; ++c) {
-        int o = d.chain_off[c], n = d.chain_off[c + 1] - o;
-        for (int k = 1 + g.lane; k <= n - 2; k += TPW) part += d.k_bend * bend_term(pos, o, k);
-        for (int j = g.lane; j <= n - 4; j += TPW) part -= d.k_tors * torsion_term(pos, o, j);
-        if (d.k_fene != 0.0)
-            for (int l = g.lane; l <= n - 2; l += TPW) part += fene_term(d, pos, o, l);
-    }
+// Full energy with the Lennard-Jones pairs in FP32 (from the working copy; each lane's row sums
+// added in double-float) and the local terms in FP64 (from x64).
+static __device__ double full_energy_working32(const SysDesc& d, const double* x64, const Slot<float>& s, const Group<32>& g) {
+    using PT = float;
+    double part = local_energy64_warp(d, x64, g.lane, 0, 1);
     const PT L = (PT)d.box_L, iL = (PT)d.inv_L;
+    DF rows{0.0f, 0.0f};
     for (int i = 0; i < d.N; ++i) {
         const P4<PT> a = s.r[i];
         const int ci = a.tag >> 1, si = a.tag & 1;
         PT row = (PT)0;
-        for (int j = i + 1 + g.lane; j < d.N; j += TPW) {
+        for (int j = i + 1 + g.lane; j < d.N; j += 32) {
             const P4<PT> b = s.r[j];
             const int cj = b.tag >> 1;
             if (ci == cj && j < i + 2) continue;
@@ -1471,10 +1499,11 @@ __device__ double full_energy_working(const SysDesc& d, const double* x64, const
                 dx += sh.x; dy += sh.y; dz += sh.z;
                 Lj = L; iLj = iL;
             }
-            PT e = lj_pair<PT>(dx, dy, dz, Lj, iLj, (PT)d.C[2 * si + (b.tag & 1)]);
-            row += (ci == cj ? (PT)d.k_lj_intra : (PT)d.k_lj_inter) * e;
+            PT e = lj_pair<PT>(dx, dy, dz, Lj, iLj, d.C32[2 * si + (b.tag & 1)]);
+            row += (ci == cj ? d.kin32 : d.kout32) * e;
         }
-        part += (double)row;
+        rows = df_add(rows, DF{row, 0.0f});
     }
+    part += f32_to_f64(rows.hi) + f32_to_f64(rows.lo);
     return g.sum(part);
 }

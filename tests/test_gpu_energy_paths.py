@@ -1,0 +1,64 @@
+"""FP64 energies around the edges of their two paths: system sizes about the smallest that takes far pairs in
+double-float, boxes so small that many image counts are not settled in FP32, pairs at the distance where the paths part,
+coordinates far from the origin, chains of every mix.  Tolerance: the suite's 1e-11 for FP64 energies."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1702_01770_gb300 import inputs
+from helpers import oracle_model, random_conformations
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def phast():
+    from paper_1702_01770_gb300 import phast
+    phast.lib()
+    return phast
+
+
+def _system(lens, L, k_tors=-0.5):
+    rng = np.random.Generator(np.random.Philox(17))
+    seq = np.concatenate([inputs.random_sequence(n, 0.5, rng) for n in lens])
+    return inputs.System("e", np.array(lens, np.int32), seq, L, k_tors=k_tors)
+
+
+SYSTEMS = [([3], 0.0), ([4], 0.0), ([30], 0.0), ([33], 0.0), ([47], 0.0), ([48], 0.0), ([49], 0.0), ([3] * 16, 30.0), ([24, 25], 9.0),
+           ([24, 24], 8.5), ([20, 41, 3], 0.0), ([100], 0.0), ([32] * 16, 60.0)]
+
+
+@pytest.mark.parametrize("lens,L", SYSTEMS, ids=["%d-%d%s" % (len(s[0]), sum(s[0]), "p" if s[1] else "") for s in SYSTEMS])
+def test_fp64_energies_of_every_size(phast, orc, lens, L):
+    s = _system(lens, L)
+    if L == 9.0 or L == 8.5:   # too dense for the placing helper: walks laid side by side, many images on the edge
+        rng = np.random.default_rng(4)
+        x = np.stack([np.concatenate([inputs.random_saw(n, 1.0, rng) + np.array([L / 2 * i, 0.37 * i, 0.2 * i]) for i, n in enumerate(lens)])
+                      for _ in range(7)])
+    else:
+        x = random_conformations(s, 7 if sum(lens) < 300 else 2, seed=sum(lens))
+        if L == 0 and len(lens) > 1:
+            x[:, lens[0]:] += np.array([5.0, 0.0, 0.0])
+            x[:, lens[0] + lens[1]:] += np.array([0.0, 40.0, 0.0])
+    x[1] += 1.0e5                                          # far from the origin
+    E = phast.phast_energy(s, torch.from_numpy(x).cuda()).cpu().numpy()
+    m = oracle_model(orc, s)
+    ref = np.array([orc.energy(m, xb) for xb in x])
+    assert np.all(np.isfinite(ref))
+    assert np.all(np.abs(E - ref) <= 1e-11 * np.maximum(1.0, np.abs(ref))), np.abs(E - ref)
+
+
+@pytest.mark.parametrize("L", [0.0, 8.0, 25.0])
+def test_pairs_where_the_paths_part(phast, orc, L):
+    """Two straight chains set so that pairs lie at distance 4, an ulp and 1e-7 to either side, and (L = 8) on the image's
+    edge; and coincident monomers, whose energy is infinite."""
+    n = 30
+    s = _system([n, n], L, k_tors=0.0)
+    x = np.stack([np.concatenate([inputs.straight_chain(n, (0, 0, 0), (0, 0, 1)), inputs.straight_chain(n, (r, 0, 0), (0, 0, 1))])
+                  for r in (4.0, np.nextafter(4.0, 0), np.nextafter(4.0, 9), 4.0 - 1e-7, 4.0 + 1e-7, 3.0, 11.9, 12.0, 1.0e7 + 3.0)])   # (1e7 itself is a whole number of boxes of 8: coincident)
+    E = phast.phast_energy(s, torch.from_numpy(x).cuda()).cpu().numpy()
+    m = oracle_model(orc, s)
+    ref = np.array([orc.energy(m, xb) for xb in x])
+    assert np.all(np.abs(E - ref) <= 1e-11 * np.maximum(1.0, np.abs(ref))), (E, ref)
+    x[0, n:] = x[0, :n]
+    assert phast.phast_energy(s, torch.from_numpy(x[:1]).cuda()).item() == np.inf
