@@ -2,14 +2,9 @@
 // batches of conformations, and multicanonical reweighting of canonical
 // averages and their parameter derivatives (Sec. 2.2).
 //
-// phast_energy_grad: one warp per conformation on the working copy the sweep
-// uses (FP32 coordinates relative to chain centroids, or FP64).  Each lane
-// owns monomers i = lane, lane + 32, ... and gathers its whole gradient: every
-// Lennard-Jones partner j (the pair is evaluated from both ends, no atomics,
-// a deterministic order), and the bending and torsion terms that contain i.
-// Energies and parameter derivatives count each pair and term once.  Nothing
-// is stored between the forward and the backward pass: the backward pass
-// recomputes (checkpointed recomputation).
+// phast_energy_grad and the passes of a training step: one warp per conformation, in FP64 or
+// with FP32 pair terms.  No atomics, a deterministic order.  Nothing is stored between the
+// forward and the backward pass: the backward pass recomputes (checkpointed recomputation).
 #include <cooperative_groups.h>
 
 #include "exp64.cuh"
@@ -55,22 +50,6 @@ __device__ __forceinline__ Coef<PT> coef(const SysDesc& d, const double* __restr
     return Coef<PT>{(PT)d.C[0], (PT)d.C[1], (PT)d.C[2], (PT)d.C[3], (PT)d.k_tors, (PT)d.k_bend};
 }
 
-// d(1 - cos theta_k)/dx_{k-1+which}, theta_k between a = x_k - x_{k-1} and b = x_{k+1} - x_k.
-template <typename PT, class Pos>
-__device__ V3<PT> bend_grad(const Pos& pos, int o, int k, int which) {
-    const P4<PT> x0 = pos(o + k - 1), x1 = pos(o + k), x2 = pos(o + k + 1);
-    const V3<PT> a = sub3(x1, x0), b = sub3(x2, x1);
-    const PT aa = dot3(a, a), bb = dot3(b, b);
-    const PT lab = sqrt(aa) * sqrt(bb);
-    const PT cs = dot3(a, b) / lab;
-    const V3<PT> dca = axpy3(-cs / aa, a, V3<PT>{b.x / lab, b.y / lab, b.z / lab});   // d cos / d a
-    const V3<PT> dcb = axpy3(-cs / bb, b, V3<PT>{a.x / lab, a.y / lab, a.z / lab});   // d cos / d b
-    // x_{k-1}: -d cos/d a -> +dca for 1 - cos; x_k: dca - dcb -> -(dca - dcb); x_{k+1}: -dcb
-    if (which == 0) return dca;
-    if (which == 1) return V3<PT>{dcb.x - dca.x, dcb.y - dca.y, dcb.z - dca.z};
-    return V3<PT>{-dcb.x, -dcb.y, -dcb.z};
-}
-
 // d cos tau_j / dx_{j+which}: n1 = u x v, n2 = v x w from u, v, w the bonds of monomers j..j+3;
 // zero for a degenerate dihedral (|n1|^2 |n2|^2 < 1e-20), where the term is 0.
 template <typename PT, class Pos>
@@ -94,135 +73,188 @@ __device__ V3<PT> torsion_grad(const Pos& pos, int o, int j, int which) {
     return dw;
 }
 
-template <typename PT>
-__device__ __forceinline__ PT nearest_count(PT x, PT iL);
-template <>
-__device__ __forceinline__ double nearest_count<double>(double x, double iL) { return rint(x * iL); }
+// ---------------------------------------------------------------------------
+// FP64 form: one warp per conformation.  An FP64 instruction holds an SMSP's pipe for 64 to 76
+// cycles, so their number is what counts: every pair once (a lane's row i against the
+// partner s places on, cyclically; the force goes to the row's registers and, with the
+// opposite sign, to the partner's sum in shared memory -- the lanes of a step have different
+// partners), every bending and torsion term once (added to its monomers in turn), reciprocals
+// by one corrected approximation.  23 FP64 instructions a pair.  4096 conformations of a
+// 55-mer: 448 us (1200 us with both ends of a pair and the local terms of every monomer).
+// ---------------------------------------------------------------------------
+struct Grad64Slot {
+    double *x, *y, *z;      // [N] positions
+    double *gx, *gy, *gz;   // [N] gradient
+};
+__host__ __device__ inline size_t grad64_slot_bytes(int N) { return sizeof(double) * 6 * (size_t)N; }
 
-template <typename PT>
+__device__ __forceinline__ V3<double> at64(const Grad64Slot& s, int j) { return V3<double>{s.x[j], s.y[j], s.z[j]}; }
+__device__ __forceinline__ V3<double> diff64(const V3<double>& a, const V3<double>& b) { return V3<double>{a.x - b.x, a.y - b.y, a.z - b.z}; }
+__device__ __forceinline__ void add64(const Grad64Slot& s, int j, double k, const V3<double>& g) {
+    s.gx[j] += k * g.x;
+    s.gy[j] += k * g.y;
+    s.gz[j] += k * g.z;
+}
+
 __global__ void __launch_bounds__(32 * kGradWarps)
-energy_grad_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* __restrict__ E_out,
-                   double* __restrict__ grad_xyz, double* __restrict__ grad_ff, SlotLayout L,
-                   const double* __restrict__ pdev) {
+energy_grad64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* __restrict__ E_out,
+                     double* __restrict__ grad_xyz, double* __restrict__ grad_ff, const double* __restrict__ pdev) {
     extern __shared__ __align__(16) unsigned char smem[];
-    Group<32> g;
-    const int w = threadIdx.x >> 5;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int b = blockIdx.x * kGradWarps + w;
     if (b >= B) return;
-    const double* x64 = xyz + (size_t)b * d.N * 3;
-    Slot<PT> s(smem + (size_t)w * L.bytes, L);
-    build_working<32, PT>(d, x64, s, g);
-    auto pos = [&](int j) -> P4<PT> { return s.r[j]; };
-    const FF<PT> f{d};
-    const Coef<PT> cf = coef<PT>(d, pdev);
-    const int nc = d.n_chains;
-    const PT Lb = f.L(), iLb = f.iL();
-    double E = 0.0, gp[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-
-    // bending and torsion energies, each term once
+    const int N = d.N, nc = d.n_chains;
+    double* base = reinterpret_cast<double*>(smem) + (size_t)w * 6 * N;
+    const Grad64Slot s{base, base + N, base + 2 * N, base + 3 * N, base + 4 * N, base + 5 * N};
+    const double* x64 = xyz + (size_t)b * N * 3;
+    bool out = false;   // a monomer beyond the container's wall: infinite energy
+    for (int j = lane; j < N; j += 32) {
+        const double3 p = ld3(x64 + 3 * j);
+        s.x[j] = p.x; s.y[j] = p.y; s.z[j] = p.z;
+        s.gx[j] = s.gy[j] = s.gz[j] = 0.0;
+        if (d.has_sphere) out |= !inside64(d, p);
+    }
+    __syncwarp();
+    const Coef<double> cf = coef<double>(d, pdev);
+    // E, sum 1 - cos theta, -sum cos tau, and minus the sums of k s^3 over AA, BB and AB pairs
+    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int c = 0; c < nc; ++c) {
         const int o = d.chain_off[c], n = d.chain_off[c + 1] - o;
-        for (int k = 1 + g.lane; k <= n - 2; k += 32) {
-            const double t = (double)bend_w<PT>(pos, o, k);
-            gp[4] += t;
-            E += (double)cf.kb * t;
-        }
-        for (int j = g.lane; j <= n - 4; j += 32) {
-            const double t = (double)torsion_w<PT>(pos, o, j);
-            gp[3] -= t;
-            E -= (double)cf.kt * t;
-        }
-        if (d.k_fene != 0.0)
-            for (int l = g.lane; l <= n - 2; l += 32) E += (double)fene_w<PT>(d, pos, o, l);
-    }
-    bool out = false;   // a monomer beyond the container's wall: infinite energy
-    for (int j = g.lane; j < d.N; j += 32) out |= !inside64(d, ld3(x64 + 3 * j));
-    // each lane's monomers: Lennard-Jones partners, then its local terms
-    for (int i = g.lane; i < d.N; i += 32) {
-        const P4<PT> a = s.r[i];
-        const int ci = a.tag >> 1, si = a.tag & 1;
-        PT gx = 0, gy = 0, gz = 0;
-        PT e_i = 0, p_aa = 0, p_bb = 0, p_ab = 0;
-        for (int j = 0; j < d.N; ++j) {
-            const P4<PT> q = s.r[j];
-            const int cj = q.tag >> 1;
-            if (j == i || (ci == cj && (j == i - 1 || j == i + 1))) continue;
-            PT dx = a.x - q.x, dy = a.y - q.y, dz = a.z - q.z;
-            PT k = f.kin();
-            if (ci != cj) {
-                const P4<PT> sh = s.D[ci * nc + cj];
-                dx += sh.x; dy += sh.y; dz += sh.z;
-                if (d.box_L > 0.0) {
-                    dx -= Lb * nearest_count<PT>(dx, iLb);
-                    dy -= Lb * nearest_count<PT>(dy, iLb);
-                    dz -= Lb * nearest_count<PT>(dz, iLb);
-                }
-                k = f.kout();
+        for (int k0 = 1; k0 <= n - 2; k0 += 32) {
+            const int k = o + k0 + lane;
+            const bool on = k0 + lane <= n - 2;
+            V3<double> ga{0, 0, 0}, gb{0, 0, 0};   // d cos / d a, d cos / d b for bonds a, b
+            if (on) {
+                const V3<double> x1 = at64(s, k), u = diff64(x1, at64(s, k - 1)), t = diff64(at64(s, k + 1), x1);
+                const double aa = dot3(u, u), bb = dot3(t, t);
+                const double il = rsqrt64(aa * bb), cs = dot3(u, t) * il;
+                const double ia = cs * rcp64(aa), ib = cs * rcp64(bb);
+                ga = V3<double>{t.x * il - ia * u.x, t.y * il - ia * u.y, t.z * il - ia * u.z};
+                gb = V3<double>{u.x * il - ib * t.x, u.y * il - ib * t.y, u.z * il - ib * t.z};
+                v[1] += 1.0 - cs;
             }
-            const int sj = q.tag & 1;
-            const PT C = cf.c(2 * si + sj);
-            const PT sv = (PT)1 / (dx * dx + dy * dy + dz * dz);
-            const PT s3 = sv * sv * sv, s6 = s3 * s3;
-            const PT fr = (PT)2 * k * sv * ((PT)3 * C * s3 - (PT)6 * s6);   // 2 dphi/d(r^2)
-            gx += fr * dx;
-            gy += fr * dy;
-            gz += fr * dz;
-            if (i < j) {
-                e_i += k * (s6 - C * s3);
-                const PT t = k * s3;
-                if (si != sj) p_ab -= t;
-                else if (si == 0) p_aa -= t;
-                else p_bb -= t;
+            if (grad_xyz) {   // 1 - cos: +ga, gb - ga, -gb
+                if (on) add64(s, k - 1, cf.kb, ga);
+                __syncwarp();
+                if (on) add64(s, k, cf.kb, diff64(gb, ga));
+                __syncwarp();
+                if (on) add64(s, k + 1, -cf.kb, gb);
+                __syncwarp();
             }
         }
-        E += (double)e_i;
-        gp[0] += (double)p_aa;
-        gp[1] += (double)p_bb;
-        gp[2] += (double)p_ab;
-        if (grad_xyz) {
-            const int o = d.chain_off[ci], n = d.chain_off[ci + 1] - o, li = i - o;
-            for (int k = li - 1; k <= li + 1; ++k) {   // bends containing i
-                if (k < 1 || k > n - 2) continue;
-                const V3<PT> t = bend_grad<PT>(pos, o, k, li - (k - 1));
-                gx += cf.kb * t.x;
-                gy += cf.kb * t.y;
-                gz += cf.kb * t.z;
-            }
-            for (int j = li - 3; j <= li; ++j) {       // dihedrals containing i: -kappa cos tau
-                if (j < 0 || j > n - 4) continue;
-                const V3<PT> t = torsion_grad<PT>(pos, o, j, li - j);
-                gx -= cf.kt * t.x;
-                gy -= cf.kt * t.y;
-                gz -= cf.kt * t.z;
-            }
-            if (d.k_fene != 0.0) {   // bonds of i: d/dr [k R^2 C_F ln(1 - x^2)] = -2 k R C_F x / (1 - x^2)
-                for (int l = li - 1; l <= li; ++l) {
-                    if (l < 0 || l > n - 2) continue;
-                    const V3<PT> b = sub3(s.r[o + l + 1], s.r[o + l]);
-                    const PT r = sqrt(dot3(b, b));
-                    const PT R = (PT)d.fene_R;
-                    const PT x = (r - (PT)d.fene_r0) / R;
-                    const PT cf = (PT)d.C_F[2 * d.seq[o + l] + d.seq[o + l + 1]];
-                    const PT dphi = (PT)(-2.0 * d.k_fene) * R * cf * x / ((PT)1 - x * x);
-                    const PT sg = (l == li) ? (PT)-1 : (PT)1;   // i is the bond's first or second monomer
-                    gx += sg * dphi * b.x / r;
-                    gy += sg * dphi * b.y / r;
-                    gz += sg * dphi * b.z / r;
+        for (int j0 = 0; j0 <= n - 4; j0 += 32) {
+            const int j = o + j0 + lane;
+            const bool on = j0 + lane <= n - 4;
+            V3<double> du{0, 0, 0}, dv{0, 0, 0}, dw{0, 0, 0};   // d cos tau by the three bonds
+            if (on) {
+                const V3<double> x0 = at64(s, j), x1 = at64(s, j + 1), x2 = at64(s, j + 2), x3 = at64(s, j + 3);
+                const V3<double> u = diff64(x1, x0), t = diff64(x2, x1), q = diff64(x3, x2);
+                const V3<double> n1 = cross3(u, t), n2 = cross3(t, q);
+                const double n11 = dot3(n1, n1), n22 = dot3(n2, n2), p = n11 * n22;
+                if (!(p < 1e-20)) {   // a degenerate dihedral has no term
+                    const double il = rsqrt64(p), cs = dot3(n1, n2) * il;
+                    const double c1 = cs * rcp64(n11), c2 = cs * rcp64(n22);
+                    const V3<double> g1{n2.x * il - c1 * n1.x, n2.y * il - c1 * n1.y, n2.z * il - c1 * n1.z};
+                    const V3<double> g2{n1.x * il - c2 * n2.x, n1.y * il - c2 * n2.y, n1.z * il - c2 * n2.z};
+                    du = cross3(t, g1);
+                    dv = axpy3(1.0, cross3(g1, u), cross3(q, g2));
+                    dw = cross3(g2, t);
+                    v[2] -= cs;
                 }
             }
-            double* out = grad_xyz + ((size_t)b * d.N + i) * 3;
-            out[0] = (double)gx;
-            out[1] = (double)gy;
-            out[2] = (double)gz;
+            if (grad_xyz) {   // -kappa cos tau: monomers get -du, du - dv, dv - dw, dw
+                if (on) add64(s, j, cf.kt, du);
+                __syncwarp();
+                if (on) add64(s, j + 1, -cf.kt, diff64(du, dv));
+                __syncwarp();
+                if (on) add64(s, j + 2, -cf.kt, diff64(dv, dw));
+                __syncwarp();
+                if (on) add64(s, j + 3, -cf.kt, dw);
+                __syncwarp();
+            }
         }
+        if (d.k_fene != 0.0)   // bond l: d/dr [k R^2 C_F ln(1 - x^2)] = -2 k R C_F x / (1 - x^2)
+            for (int l0 = 0; l0 <= n - 2; l0 += 32) {
+                const int l = o + l0 + lane;
+                const bool on = l0 + lane <= n - 2;
+                V3<double> u{0, 0, 0};
+                double dphi = 0.0;
+                if (on) {
+                    v[0] += fene_term(d, [&](int j) { return make_double3(s.x[j], s.y[j], s.z[j]); }, l, 0);
+                    const V3<double> q = diff64(at64(s, l + 1), at64(s, l));
+                    const double r = sqrt(dot3(q, q)), x = (r - d.fene_r0) / d.fene_R;
+                    dphi = -2.0 * d.k_fene * d.fene_R * d.C_F[2 * d.seq[l] + d.seq[l + 1]] * x / (1.0 - x * x);
+                    u = V3<double>{q.x / r, q.y / r, q.z / r};
+                }
+                if (grad_xyz) {
+                    if (on) add64(s, l, -dphi, u);
+                    __syncwarp();
+                    if (on) add64(s, l + 1, dphi, u);
+                    __syncwarp();
+                }
+            }
     }
-    E = g.sum(E);
-    if (__any_sync(g.mask, out)) E = INFINITY;
-    for (int q = 0; q < 5; ++q) gp[q] = g.sum(gp[q]);
-    if (g.lane == 0) {
-        if (E_out) E_out[b] = E;
-        if (grad_ff)
-            for (int q = 0; q < 5; ++q) grad_ff[(size_t)b * 5 + q] = gp[q];
+    v[0] += cf.kb * v[1] + cf.kt * v[2];
+    for (int i0 = 0; i0 < N; i0 += 32) {
+        const int i = i0 + lane;
+        const bool row = i < N;
+        const V3<double> a = at64(s, row ? i : 0);
+        const int ci = row ? d.chain_of[i] : 0, si = row ? d.seq[i] : 0;
+        V3<double> g{0, 0, 0};
+        for (int m = 1; 2 * m <= N; ++m) {
+            int j = i + m;
+            if (j >= N) j -= N;
+            // every pair once (opposite places from the first half); bonded pairs have no term
+            const bool on = row && !(2 * m == N && 2 * i >= N) && !(m == 1 && j == i + 1 && d.chain_of[j] == ci);
+            if (on) {
+                const bool inter = d.chain_of[j] != ci;
+                const int sj = d.seq[j];
+                V3<double> q = diff64(a, at64(s, j));
+                if (inter) {
+                    q.x = mimage64_short(d, q.x);
+                    q.y = mimage64_short(d, q.y);
+                    q.z = mimage64_short(d, q.z);
+                }
+                const double k = inter ? d.k_lj_inter : d.k_lj_intra, C = cf.c(2 * si + sj);
+                const double sv = rcp64(dot3(q, q)), s2 = sv * sv, s3 = s2 * sv, ks3 = k * s3;
+                v[0] = __fma_rn(ks3, s3 - C, v[0]);   // k (s^6 - C s^3)
+                const int cls = si == sj ? 3 + si : 5;
+                const double sum = (cls == 3 ? v[3] : cls == 4 ? v[4] : v[5]) - ks3;
+                v[3] = cls == 3 ? sum : v[3];
+                v[4] = cls == 4 ? sum : v[4];
+                v[5] = cls == 5 ? sum : v[5];
+                if (grad_xyz) {
+                    const double fr = ks3 * sv * __fma_rn(-12.0, s3, 6.0 * C);   // 2 dphi/d(r^2)
+                    g.x = __fma_rn(fr, q.x, g.x);
+                    g.y = __fma_rn(fr, q.y, g.y);
+                    g.z = __fma_rn(fr, q.z, g.z);
+                    s.gx[j] = __fma_rn(-fr, q.x, s.gx[j]);
+                    s.gy[j] = __fma_rn(-fr, q.y, s.gy[j]);
+                    s.gz[j] = __fma_rn(-fr, q.z, s.gz[j]);
+                }
+            }
+            __syncwarp();
+        }
+        if (row && grad_xyz) {
+            s.gx[i] += g.x;
+            s.gy[i] += g.y;
+            s.gz[i] += g.z;
+        }
+        __syncwarp();
+    }
+    if (grad_xyz)
+        for (int e = lane; e < 3 * N; e += 32) {
+            const int j = e / 3, q = e - 3 * j;
+            grad_xyz[(size_t)b * N * 3 + e] = (q == 0 ? s.gx : q == 1 ? s.gy : s.gz)[j];
+        }
+    out = __any_sync(full, out);
+    int first = 0, count = 6;
+    warp_sums<6>(v, &first, &count);
+    if (count == 1) {
+        if (first == 0 && E_out) E_out[b] = out ? INFINITY : v[0];
+        // v[1..5]: kappa_C, kappa, AA, BB, AB -> columns 4, 3, 0, 1, 2
+        if (first > 0 && grad_ff) grad_ff[(size_t)b * 5 + (first == 1 ? 4 : first == 2 ? 3 : first - 3)] = v[0];
     }
 }
 
@@ -1024,10 +1056,9 @@ int energy_grad(const phast_system* sys, const phast_ff* ff, int32_t B, const do
     cudaStream_t st = (cudaStream_t)stream;
     if (pair_precision == 64) {
         dim3 grid((B + kGradWarps - 1) / kGradWarps), block(32 * kGradWarps);
-        SlotLayout L = slot_layout<double>(d.N, d.n_chains, d.max_chain);
-        size_t sm = (size_t)L.bytes * kGradWarps;
-        PHAST_CUDA_TRY(cudaFuncSetAttribute(energy_grad_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        energy_grad_kernel<double><<<grid, block, sm, st>>>(d, B, xyz, E_out, grad_xyz, grad_ff, L, params);
+        const size_t sm = grad64_slot_bytes(d.N) * kGradWarps;
+        PHAST_CUDA_TRY(cudaFuncSetAttribute(energy_grad64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        energy_grad64_kernel<<<grid, block, sm, st>>>(d, B, xyz, E_out, grad_xyz, grad_ff, params);
         PHAST_CUDA_TRY(cudaGetLastError());
         return PHAST_OK;
     }
