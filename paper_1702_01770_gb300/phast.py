@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from dataclasses import dataclass
 
 import numpy as np
@@ -131,8 +132,13 @@ def _check(rc: int):
         raise PhastError(rc, lib().phast_last_error().decode())
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # without building a Stream object
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
@@ -183,9 +189,24 @@ class _Structs:
             self.mp[i].pair_precision = int(pair_precision or 64)
 
 
+class _CallStructs:
+    """The system and force-field structs of one energy call, packed in one go (the ABI structs of _Structs
+    without the multicanonical set-up; the arrays are kept until the call returns)."""
+    __slots__ = ("keep", "sys", "ff")
+
+    def __init__(self, s):
+        cl = np.ascontiguousarray(s.chain_len, dtype=np.int32)
+        sq = np.ascontiguousarray(s.seq, dtype=np.uint8)
+        self.keep = (cl, sq)
+        self.sys = _System.from_buffer_copy(struct.pack("@iPPdd", cl.size, cl.__array_interface__["data"][0],
+                                                        sq.__array_interface__["data"][0], s.box_L, s.sphere_R))
+        self.ff = _FF.from_buffer_copy(struct.pack("@15d", s.k_bend, s.k_tors, s.k_lj_intra, s.k_lj_inter, *s.C,
+                                                   s.k_fene, s.fene_r0, s.fene_R, *s.C_F))
+
+
 def phast_energy(system, xyz: torch.Tensor, pair_precision: int = 64, stream=None) -> torch.Tensor:
     """Energies (FP64, device) of xyz [B, N, 3] FP64 on the device."""
-    st = _Structs([system])
+    st = _CallStructs(system)
     xyz = xyz.contiguous()
     B = xyz.shape[0] if xyz.numel() else 0
     E = torch.empty(B, dtype=torch.float64, device=xyz.device)
@@ -214,7 +235,7 @@ def phast_energy_grad(system, xyz: torch.Tensor, pair_precision: int = 32, want_
     """(E [B], dE/dxyz [B, N, 3] or None, dE/d(C_AA, C_BB, C_AB, kappa, kappa_C) [B, 5] or None),
     FP64 on the device, of xyz [B, N, 3] FP64 on the device.  params: FP64 [5] on the device
     (ff_params order) in place of the system's values (phast_energy_grad_params)."""
-    st = _Structs([system])
+    st = _CallStructs(system)
     xyz = xyz.contiguous()
     B = xyz.shape[0] if xyz.numel() else 0
     E = torch.empty(B, dtype=torch.float64, device=xyz.device)
@@ -255,7 +276,7 @@ class EnergyFunction(torch.autograd.Function):
         ctx.system, ctx.pair_precision = system, pair_precision
         if pair_precision == 32 and xyz.dtype in _BITS:
             x, p = xyz.contiguous(), _device_params(params, xyz)
-            ctx.structs = st = _Structs([system])
+            ctx.structs = st = _CallStructs(system)
             B = x.shape[0] if x.numel() else 0
             E = torch.empty(B, dtype=torch.float64, device=x.device)
             _check(lib().phast_energy_forward32(st.sys, st.ff, B, _ptr(x), _BITS[x.dtype], _ptr(p), _BITS[p.dtype],
@@ -318,7 +339,7 @@ def moves_tensor(moves, device) -> torch.Tensor:
 
 def phast_delta_energy(system, xyz: torch.Tensor, moves, pair_precision: int = 64, want_xyz: bool = False,
                        stream=None):
-    st = _Structs([system])
+    st = _CallStructs(system)
     xyz = xyz.contiguous()
     B = xyz.shape[0]
     mv = moves if isinstance(moves, torch.Tensor) else moves_tensor(moves, xyz.device)
@@ -544,7 +565,7 @@ def phast_micro_analysis(lnW: torch.Tensor, e_min: float, bin_width: float, hist
     if T is None:
         T = torch.empty(0, dtype=torch.float64, device=dev)
     n_T = T.numel()
-    f = lambda n: torch.full((n,), float("nan"), dtype=torch.float64, device=dev)
+    f = lambda n: torch.empty(n, dtype=torch.float64, device=dev)   # every element is written
     errs = n_blocks >= 2
     r = MicroResult(f(K), f(K), f(K), f(n_T), f(n_T), f(2))
     if errs:
@@ -565,7 +586,8 @@ def _micro_out(r: MicroResult) -> _MicroOut:
     o = _MicroOut()
     for name in _MicroOut._fields_:
         v = getattr(r, name[0])
-        setattr(o, name[0], None if v is None else v.data_ptr())
+        if v is not None:
+            setattr(o, name[0], v.data_ptr())
     return o
 
 
@@ -595,7 +617,7 @@ def phast_micro_analysis_binned(lnW: torch.Tensor, e_min: float, bin_width: floa
     if T is None:
         T = torch.empty(0, dtype=torch.float64, device=dev)
     n_T = T.numel()
-    f = lambda n: torch.full((n,), float("nan"), dtype=torch.float64, device=dev)
+    f = lambda n: torch.empty(n, dtype=torch.float64, device=dev)   # every element is written
     r = MicroResult(f(K), f(K), f(K), f(n_T), f(n_T), f(2))
     r.S_err, r.beta_err, r.CV_err, r.E_T_err, r.cV_T_err, r.peak_err = f(K), f(K), f(K), f(n_T), f(n_T), f(2)
     o = _MicroOut()
