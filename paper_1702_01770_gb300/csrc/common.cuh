@@ -254,17 +254,30 @@ __device__ __forceinline__ bool marsaglia_try(uint4 r, double3* axis) {
 // Centroid of monomers o..o+n-1 in the fixed summation order of the move's
 // specification: 32 strided partial sums s_l over j = l, l+32, ... (increasing
 // j), halved by s_l += s_{l+w} for w = 16, 8, 4, 2, 1, then s_0 / n.  One thread.
-__device__ __forceinline__ double3 centroid_serial(const double* x64, int o, int n) {
+// The additions of partial sums beyond the chain (zeros) are left out.
+__device__ __forceinline__ double3 centroid_serial(const SysDesc& d, const double* x64, int ch) {
+    const int o = d.chain_off[ch], n = d.chain_off[ch + 1] - o;
     double c[3];
-    for (int d = 0; d < 3; ++d) {
-        double part[32];
-        for (int l = 0; l < 32; ++l) {
+    for (int k = 0; k < 3; ++k) {
+        const double* x = x64 + 3 * o + k;
+        auto strided = [&](int l) {
+            double p = x[3 * l];
+            for (int j = l + 32; j < n; j += 32) p = xadd(p, x[3 * j]);
+            return p;
+        };
+        double part[16];   // after the step w = 16
+#pragma unroll
+        for (int l = 0; l < 16; ++l) {
             part[l] = 0.0;
-            for (int j = l; j < n; j += 32) part[l] = xadd(part[l], x64[3 * (o + j) + d]);
+            if (l < n) part[l] = strided(l);
+            if (l + 16 < n) part[l] = xadd(part[l], strided(l + 16));
         }
-        for (int w = 16; w >= 1; w /= 2)
-            for (int l = 0; l < w; ++l) part[l] = xadd(part[l], part[l + w]);
-        c[d] = xdiv(part[0], (double)n);
+#pragma unroll
+        for (int w = 8; w >= 1; w /= 2)
+#pragma unroll
+            for (int l = 0; l < w; ++l)
+                if (l + w < n) part[l] = xadd(part[l], part[l + w]);
+        c[k] = div_count(part[0], count_to_f64(n), d.inv_len[ch]);
     }
     return make_double3(c[0], c[1], c[2]);
 }
@@ -445,7 +458,10 @@ __device__ __forceinline__ bool bond_step(const Pos& pos, int o, int n, int l, d
 
 // Steric container (hard wall about the origin): true if (x^2 + y^2) + z^2 <= R^2.
 __device__ __forceinline__ bool inside64(const SysDesc& d, double3 x) {
-    return !(d.sphere_R2 > 0.0) || xadd(xadd(xmul(x.x, x.x), xmul(x.y, x.y)), xmul(x.z, x.z)) <= d.sphere_R2;
+    // non-negative values order as their bit patterns, a NaN (either sign) above all
+    const double r2 = xadd(xadd(xmul(x.x, x.x), xmul(x.y, x.y)), xmul(x.z, x.z));
+    return !d.has_sphere ||
+           (__double_as_longlong(r2) & 0x7fffffffffffffffll) <= __double_as_longlong(d.sphere_R2);
 }
 
 // Lennard-Jones pair of Eq. 2/3 without its coupling: r^-12 - C r^-6 (FP64).
@@ -498,6 +514,23 @@ __device__ __forceinline__ double rsqrt64(double x) {
     const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
     return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
 }
+// Change of the FENE term of bond l between two configurations, as one logarithm of a
+// quotient (an FP64 logarithm takes 2100 cycles a warp): +inf, or NaN from an infinite
+// start, where fene_term's difference is.
+template <class PosA, class PosB>
+__device__ __forceinline__ double fene_change(const SysDesc& d, const PosA& before, const PosB& after, int o, int l) {
+    auto rest = [&](double3 a, double3 b) -> double {   // 1 - ((r - r0) / R)^2
+        const double dx = b.x - a.x, dy = b.y - a.y, dz = b.z - a.z;
+        const double x = (sqrt((dx * dx + dy * dy) + dz * dz) - d.fene_r0) / d.fene_R;   // as in fene_term
+        return 1.0 - x * x;
+    };
+    const double u = rest(before(o + l), before(o + l + 1)), v = rest(after(o + l), after(o + l + 1));
+    const double k = d.fene_kR2 * d.C_F[2 * d.seq[o + l] + d.seq[o + l + 1]];
+    if (!(v > 0.0)) return u > 0.0 ? INFINITY : __longlong_as_double(0x7ff8000000000000ll);
+    if (!(u > 0.0)) return -INFINITY;
+    return k * log(v * rcp64(u));
+}
+
 __device__ __forceinline__ double flip_sign(double x, bool flip) {
     return __hiloint2double(__double2hiint(x) ^ (flip ? (int)0x80000000 : 0), __double2loint(x));
 }

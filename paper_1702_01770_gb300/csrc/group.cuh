@@ -111,16 +111,18 @@ __host__ __device__ inline SlotLayout slot_layout(int N, int nc, int mc) {
 
 // Per-warp shared-memory layout of the one-walker-per-thread sweep (bytes).
 struct LaneLayout {
-    int r_off, w_off, org_off, bytes;
+    int r_off, w_off, org_off, newr_off, bytes;
 };
+// shared_trials: the trial records of the moved monomers lie here too (else in the walkers'
+// global scratch).
 template <typename PT>
-__host__ __device__ inline LaneLayout lane_layout(int N, int nc, int mc) {
+__host__ __device__ inline LaneLayout lane_layout(int N, int nc, int mc, bool shared_trials) {
     LaneLayout L;
     int o = 0;
-    (void)mc;
     L.r_off = o;    o += 32 * (int)sizeof(P4<PT>) * N;
     L.w_off = o;    o += 32 * 16 * nc;
     L.org_off = o;  o += 32 * 16 * nc;
+    L.newr_off = o; o += shared_trials ? 32 * (int)sizeof(P4<PT>) * mc : 0;
     L.bytes = o;
     return L;
 }

@@ -19,26 +19,33 @@
 //   * walker arrays in shared memory are lane-interleaved (element e of lane l
 //     at e * 32 + l), so the lanes of a warp reach theirs without bank
 //     conflicts whatever indices they use; the FP64 master coordinates stay in
-//     global memory (L2-resident for these sizes), the trial positions (FP64
-//     and their working-precision records) in a per-walker global scratch, so
-//     that shared memory holds only the working copy and more warps fit.
+//     global memory (L2-resident for these sizes), the FP64 trial positions in a
+//     per-walker global scratch, their FP32 records in shared memory where the
+//     warps still fit (SH), else beside them.
+//
+// What bounds it: the length of a move's chain of dependent instructions (a warp takes
+// the union of its 32 walkers' paths: six proposals, the FP64 geometry, the pair loop) and
+// the instruction cache, with one warp per scheduler; 16,384 walkers of two 13-mers in a
+// sphere, 1 x 128 tiles, 10 sweeps: 25.6 ms with a branchy pair loop that gathered its
+// trial records from global memory, FP64 wall and disc tests and seven warps of seven
+// lanes per scheduler; 15.1 ms now.
 #pragma once
 
 #include "group.cuh"
 
 // One lane's view of its walker's shared arrays.
-template <typename PT>
+template <typename PT, bool SH>
 struct LaneSlot {
     P4<PT>* r;       // [N][32] working positions (FP32: relative to the chain origin; FP64: absolute)
-    P4<PT>* newr;    // [mc] trial positions of the moved monomers (the walker's global scratch)
+    P4<PT>* newr;    // trial positions of the moved monomers: [mc][32] (SH), or [mc] in the walker's global scratch
     float4* w;       // [nc][32] shift of each chain's origin from chain 0's, wrapped into the box (FP32 mode)
     float4* org;     // [nc][32] chain origins (FP32 values, exact in FP64)
     int lane;
     __device__ __forceinline__ LaneSlot(unsigned char* warp_base, const LaneLayout& L, int lane_)
-        : r((P4<PT>*)(warp_base + L.r_off)), newr(nullptr),
+        : r((P4<PT>*)(warp_base + L.r_off)), newr(SH ? (P4<PT>*)(warp_base + L.newr_off) : nullptr),
           w((float4*)(warp_base + L.w_off)), org((float4*)(warp_base + L.org_off)), lane(lane_) {}
     __device__ __forceinline__ P4<PT>& R(int j) const { return r[j * 32 + lane]; }
-    __device__ __forceinline__ P4<PT>& NR(int q) const { return newr[q]; }
+    __device__ __forceinline__ P4<PT>& NR(int q) const { return SH ? newr[q * 32 + lane] : newr[q]; }
     __device__ __forceinline__ float4& W(int c) const { return w[c * 32 + lane]; }
     __device__ __forceinline__ float4& O(int c) const { return org[c * 32 + lane]; }
 };
@@ -88,8 +95,8 @@ __device__ __forceinline__ double3 lane_origin(const double* x64, int o, int n) 
 // shift w_c = o_c - o_0 (wrapped into the box for a periodic system, exact in
 // FP64 and then rounded) and positions x - o_c rounded to FP32; FP64 mode:
 // the absolute positions.
-template <typename PT>
-__device__ void lane_build(const SysDesc& d, const double* x64, const LaneSlot<PT>& s) {
+template <typename PT, bool SH>
+__device__ void lane_build(const SysDesc& d, const double* x64, const LaneSlot<PT, SH>& s) {
     if constexpr (sizeof(PT) == 4) {
         const double3 o0 = lane_origin(x64, d.chain_off[0], d.chain_off[1] - d.chain_off[0]);
         for (int c = 0; c < d.n_chains; ++c) {
@@ -152,7 +159,7 @@ __device__ __forceinline__ bool lane_geometry(const SysDesc& d, const double* x6
     } else if (GEOM && P.type == PHAST_CAP) {
         G->c = ld3(x64 + 3 * (o + (P.index > 0 ? P.index - 1 : 1)));
     } else if (P.type == PHAST_ROT) {
-        G->c = centroid_serial(x64, o, n);
+        G->c = centroid_serial(d, x64, P.chain);
     } else {   // crankshaft about the axis through monomers i-1 and i+1
         const int i = o + P.index;
         const double3 a = ld3(x64 + 3 * (i - 1)), b = ld3(x64 + 3 * (i + 1));
@@ -171,35 +178,35 @@ __device__ __forceinline__ bool lane_geometry(const SysDesc& d, const double* x6
 
 // Lennard-Jones change of the move: every (moved, unmoved) pair, old and new
 // positions side by side in paired FP32 instructions, as one flat loop over the
-// m x U pairs (the lanes of a warp then run max(m U) iterations rather than
-// max(m) x max(U)).  Partners of other chains are taken into the moved chain's
-// frame by the difference of the chains' wrapped origin shifts and get the
-// per-pair minimum image; left-out partners contribute nothing.  Returns the
-// change with the couplings k_lj_intra / k_lj_inter applied.
-template <bool PBC>
-__device__ __forceinline__ float lane_pairs32(const SysDesc& d, const MoveSet& M, int mchain, const LaneSlot<float>& s) {
-    const int m = M.hi - M.lo + 1, U = d.N - m;
-    const int total = m * U;
+// pairs (the lanes of a warp then run max(m U) iterations rather than
+// max(m) x max(U)), summed in pair order.  The partners left out lie next to the
+// moved range (move_set), so the partners are the monomers outside one block.
+// With about one warp on an SMSP the loop is bound by the latency of its loads: every
+// iteration reads its three records from shared memory at computed places, without
+// branches, so that those of unrolled iterations overlap (16,384 walkers, 4 sweeps, 1 x 32
+// tiles: unrolled 1, 2, 4 times 7.86, 7.81, 8.40 ms; the larger body leaves the instruction cache).  Partners of other chains are
+// taken into the moved chain's frame by the difference of the chains' wrapped origin
+// shifts and get the per-pair minimum image.  Returns the change with the couplings
+// k_lj_intra / k_lj_inter applied.
+template <bool PBC, bool SH>
+__device__ __forceinline__ float lane_pairs32(const SysDesc& d, const MoveSet& M, int mchain, const LaneSlot<float, SH>& s) {
+    int lo = M.lo, hi = M.hi;
+    if (M.ex1 >= 0 || (M.ex0 >= 0 && M.ex0 < M.lo)) --lo;
+    if (M.ex2 >= 0 || M.ex0 > M.hi) ++hi;
+    const int m = M.hi - M.lo + 1, total = m * (d.N - (hi - lo + 1));
+    const int first = lo > 0 ? 0 : hi + 1;
     const float2 Mg = make_float2(12582912.0f, 12582912.0f), nMg = make_float2(-12582912.0f, -12582912.0f);
     const float4 wm = s.W(mchain);
     float acc = 0.0f;
-    int q = 0, t = 0;
-    P4<float> ow = s.R(M.lo), nw = s.NR(0);
+    int q = 0, j = first;
 #pragma unroll 2
     for (int k = 0; k < total; ++k) {
-        const int j = t < M.lo ? t : t + m;
-        const bool skip = (j == M.ex0) | (j == M.ex1) | (j == M.ex2);
-        const P4<float> p = s.R(j);
+        const P4<float> ow = s.R(M.lo + q), nw = s.NR(q), p = s.R(j);
         const int cj = p.tag >> 1;
         const float C = d.C32[2 * (ow.tag & 1) + (p.tag & 1)];
-        float qx = p.x, qy = p.y, qz = p.z;
         const bool inter = cj != mchain;
-        if (inter) {   // into the moved chain's frame
-            const float4 wc = s.W(cj);
-            qx += wc.x - wm.x;
-            qy += wc.y - wm.y;
-            qz += wc.z - wm.z;
-        }
+        const float4 wc = s.W(cj);   // into the moved chain's frame (wc = wm within the chain)
+        const float qx = p.x + (wc.x - wm.x), qy = p.y + (wc.y - wm.y), qz = p.z + (wc.z - wm.z);
         float2 dx = __fadd2_rn(make_float2(ow.x, nw.x), make_float2(-qx, -qx));
         float2 dy = __fadd2_rn(make_float2(ow.y, nw.y), make_float2(-qy, -qy));
         float2 dz = __fadd2_rn(make_float2(ow.z, nw.z), make_float2(-qz, -qz));
@@ -216,21 +223,20 @@ __device__ __forceinline__ float lane_pairs32(const SysDesc& d, const MoveSet& M
         const float2 i2 = make_float2(fast_rcp(r2.x), fast_rcp(r2.y));
         const float2 i6 = __fmul2_rn(__fmul2_rn(i2, i2), i2);
         const float2 e = __fmul2_rn(i6, __fadd2_rn(i6, make_float2(-C, -C)));
-        const float kap = skip ? 0.0f : (inter ? d.kout32 : d.kin32);
-        acc = __fmaf_rn(kap, e.y - e.x, acc);
-        if (++t == U) {   // the next moved monomer
-            t = 0;
-            if (++q < m) {
-                ow = s.R(M.lo + q);
-                nw = s.NR(q);
-            }
+        acc = __fmaf_rn(inter ? d.kout32 : d.kin32, e.y - e.x, acc);
+        ++j;
+        if (j == lo) j = hi + 1;
+        if (j >= d.N) {   // the next moved monomer
+            j = first;
+            ++q;
         }
     }
     return acc;
 }
 
 // The same in FP64 (absolute positions, per-pair minimum image between chains).
-__device__ __forceinline__ double lane_pairs64(const SysDesc& d, const MoveSet& M, int mchain, const LaneSlot<double>& s) {
+template <bool SH>
+__device__ __forceinline__ double lane_pairs64(const SysDesc& d, const MoveSet& M, int mchain, const LaneSlot<double, SH>& s) {
     const int m = M.hi - M.lo + 1, U = d.N - m;
     const int total = m * U;
     double acc = 0.0;
@@ -263,13 +269,13 @@ constexpr int kLaneRebuildSweeps = 64;
 
 // One walker, one thread: n_sweeps sweeps of the multicanonical Metropolis
 // scheme (Sec. 2.2) -- the counterpart of run_walker for a group of one lane.
-template <typename PT, bool GEOM>
-__device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id, int w_local, LaneSlot<PT> s,
+template <typename PT, bool GEOM, bool SH>
+__device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id, int w_local, LaneSlot<PT, SH> s,
                                 uint32_t* hist, unsigned long long* hist_tile, unsigned long long* hist_g) {
     const int gw = sd.walker_off + w_local;
     double* x64 = a.xyz + sd.xyz_off + (int64_t)w_local * sd.N * 3;
     double* new64 = a.scratch + (int64_t)gw * a.scratch_stride;   // the trial's exact positions [mc][3]
-    s.newr = reinterpret_cast<P4<PT>*>(new64 + 4 * sd.max_chain);   // their records [mc] (16-byte aligned)
+    if (!SH) s.newr = reinterpret_cast<P4<PT>*>(new64 + 4 * sd.max_chain);   // their records [mc] (16-byte aligned)
     const double* lnW = a.lnW + sd.lnw_off;
     double E = a.E[gw];
     int bin = a.bin[gw];
@@ -284,7 +290,10 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
     const int64_t n_moves = a.n_sweeps * sd.N;
     const uint64_t period = (uint64_t)sd.recompute_every * (uint64_t)sd.N;
     const uint64_t rebuild = (uint64_t)kLaneRebuildSweeps * (uint64_t)sd.N;
-    lane_build<PT>(sd, x64, s);
+    // moves until the next look at the two periods (64-bit remainders take about a hundred instructions each)
+    auto look = [&]() -> uint32_t { return min(moves_to_period(t, period), moves_to_period(t, rebuild)); };
+    uint32_t left = look();
+    lane_build<PT, SH>(sd, x64, s);
     double lnw_here = __ldg(lnW + bin);
     float erel = (float)(E - sd.e_min);
     for (int64_t it = 0; it < n_moves; ++it) {
@@ -293,9 +302,15 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
                        stream_block<true>(seed, t, 2u), &P);
         if constexpr (!GEOM) __builtin_assume(P.type >= 0 && P.type < PHAST_BOND);
         if (P.type == PHAST_PIVOT || P.type == PHAST_ROT || (GEOM && P.type == PHAST_CAP)) {
-            for (int j = 0; j < PHAST_MARSAGLIA_TRIES; ++j) {
-                double3 ax;
-                if (marsaglia_try(stream_block<true>(seed, t, 3u + (uint32_t)j), &ax)) { P.axis = ax; break; }
+            for (int j = 0; j < PHAST_MARSAGLIA_TRIES; ++j) {   // disc_test decides as the FP64 test
+                const uint4 blk = stream_block<true>(seed, t, 3u + (uint32_t)j);
+                float f1, f2, f3;
+                if (disc_test<false>(blk, &f1, &f2, &f3)) {
+                    double v1, v2, sd2;
+                    marsaglia_in_disc(blk, &v1, &v2, &sd2);
+                    P.axis = marsaglia_axis(v1, v2, sd2);
+                    break;
+                }
             }
         }
         const MoveSet M = move_set(sd, P.type, P.chain, P.index);
@@ -306,9 +321,10 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
         const bool ok = lane_geometry<GEOM>(sd, x64, P, &G, &jac);
         bool wall = false;
         double3 oc = make_double3(0.0, 0.0, 0.0);   // the moved chain's origin (FP32 mode)
+        float4 og = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if constexpr (sizeof(PT) == 4) {
-            const float4 og = s.O(P.chain);
-            oc = make_double3((double)og.x, (double)og.y, (double)og.z);
+            og = s.O(P.chain);
+            oc = make_double3(f32_to_f64(og.x), f32_to_f64(og.y), f32_to_f64(og.z));
         }
         if (ok) {
             for (int q = 0; q < m; ++q) {
@@ -318,14 +334,21 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
                 new64[3 * q + 0] = y.x;
                 new64[3 * q + 1] = y.y;
                 new64[3 * q + 2] = y.z;
-                if (GEOM) wall |= !inside64(sd, y);
                 P4<PT> w;
                 if constexpr (sizeof(PT) == 4) {
-                    w.x = (float)(y.x - oc.x);
-                    w.y = (float)(y.y - oc.y);
-                    w.z = (float)(y.z - oc.z);
+                    w.x = f64_to_f32(y.x - oc.x);
+                    w.y = f64_to_f32(y.y - oc.y);
+                    w.z = f64_to_f32(y.z - oc.z);
+                    if (GEOM && sd.has_sphere) {   // as container_ok: FP32 decides away from the wall
+                        const float px = og.x + w.x, py = og.y + w.y, pz = og.z + w.z;
+                        const float e = (px * px + py * py + pz * pz) - sd.sphere_R2_32;
+                        const float band = 1e-5f * sd.sphere_R2_32;
+                        if (e > band) wall = true;
+                        else if (!(e < -band)) wall |= !inside64(sd, y);
+                    }
                 } else {
                     w.x = y.x; w.y = y.y; w.z = y.z;
+                    if (GEOM) wall |= !inside64(sd, y);
                 }
                 w.tag = s.R(M.lo + q).tag;
                 s.NR(q) = w;
@@ -377,33 +400,33 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
                     auto after = [&](int j) -> double3 {
                         return (j >= M.lo && j <= M.hi) ? ld3(new64 + 3 * (j - M.lo)) : ld3(x64 + 3 * j);
                     };
-                    fene += fene_term(sd, after, o, fb0 + k) - fene_term(sd, before, o, fb0 + k);
+                    fene += fene_change(sd, before, after, o, fb0 + k);
                 }
             if constexpr (sizeof(PT) == 4) {
-                const float pr = sd.box_L > 0.0 ? lane_pairs32<true>(sd, M, P.chain, s)
-                                                : lane_pairs32<false>(sd, M, P.chain, s);
+                const float pr = sd.iL32 > 0.0f ? lane_pairs32<true, SH>(sd, M, P.chain, s)
+                                                : lane_pairs32<false, SH>(sd, M, P.chain, s);
                 dE32 = df_add(DF{loc, 0.0f}, DF{pr, 0.0f});
                 if (fene != 0.0) dE32 = df_add(dE32, df_of(fene));
             } else {
-                dE64 = loc + fene + lane_pairs64(sd, M, P.chain, s);
+                dE64 = loc + fene + lane_pairs64<SH>(sd, M, P.chain, s);
             }
         }
         const bool finite = eval && (sizeof(PT) == 4 ? (isfinite(dE32.hi) && isfinite(dE32.lo)) : isfinite(dE64));
         int b_new = -1;
-        if (finite) b_new = sizeof(PT) == 4 ? bin_after(sd, E, erel, dE32) : bin_of(sd, E + dE64);
+        if (finite) b_new = sizeof(PT) == 4 ? bin_after(sd, E, erel, dE32) : bin_of_short(sd, E + dE64);
         bool acc = false;
         double lnw_new = lnw_here;
         if (b_new >= 0) {
             lnw_new = __ldg(lnW + b_new);
             const double dl = lnw_new - lnw_here;
             if (GEOM && P.type == PHAST_BOND) acc = accept_stretch(dl, jac, P);
-            else acc = (dl >= 0.0) || accept_below(dl, P);
+            else acc = accept_weight(dl, P);
         }
         if (acc) {
-            E = E + (sizeof(PT) == 4 ? (double)dE32.hi + (double)dE32.lo : dE64);
+            E = E + (sizeof(PT) == 4 ? f32_to_f64(dE32.hi) + f32_to_f64(dE32.lo) : dE64);
             bin = b_new;
             lnw_here = lnw_new;
-            erel = (float)(E - sd.e_min);
+            erel = f64_to_f32(E - sd.e_min);
             for (int q = 0; q < m; ++q) {   // commit the exact positions and their working copy
                 x64[3 * (M.lo + q) + 0] = new64[3 * q + 0];
                 x64[3 * (M.lo + q) + 1] = new64[3 * q + 1];
@@ -435,6 +458,8 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
             a.trace[(int64_t)w_local * n_moves + it] = tr;
         }
         ++t;
+        if (--left != 0) continue;
+        left = look();
         if (period && (t % period) == 0) {   // the FP64 full energy replaces the running one
             const double Ef = lane_energy64(sd, x64);
             drift_max = fmax(drift_max, fabs(E - Ef));
@@ -447,11 +472,11 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
                 lnw_here = __ldg(lnW + bin);
                 if (bf < 0) ++n_outside;
             }
-            lane_build<PT>(sd, x64, s);   // origins re-centred, working copy rounded afresh
+            lane_build<PT, SH>(sd, x64, s);   // origins re-centred, working copy rounded afresh
         } else if (sizeof(PT) == 4 && (t % rebuild) == 0) {
             // translations carry a chain away from its origin, and its FP32 coordinates
             // lose digits: re-centre now and then even without an energy recompute
-            lane_build<PT>(sd, x64, s);
+            lane_build<PT, SH>(sd, x64, s);
         }
     }
     a.E[gw] = E;

@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kPlainThreads) sweep_plain_kernel(const SweepA
             } else if (P.type == PHAST_BOND) {
                 ok = bond_step([&](int j) { return ld3(x64 + 3 * j); }, o, n, P.index, P.angle, &step, &jac) ? 1 : 0;
             } else if (P.type == PHAST_ROT) {
-                center = centroid_serial(x64, o, n);
+                center = centroid_serial(sd, x64, P.chain);
             } else if (P.type == PHAST_CRANK) {
                 const int i = o + P.index;
                 double3 p0 = ld3(x64 + 3 * (i - 1)), p1 = ld3(x64 + 3 * (i + 1));
@@ -315,7 +315,7 @@ constexpr int kLeanMaxN = 48;
 // exact: a type with torsion starts near straight (FP32 builds without the geometry then
 // carry the exact path of the torsion terms).
 batched_fn pick_batched(int tpw, bool fp32, bool geom, bool exact, bool lean) {
-    if (tpw == 1) return pick_lane(fp32, geom);
+    if (tpw == 1) return pick_lane(fp32, geom, false);
     if (!fp32) return pick_f64(tpw, geom);
     return geom ? pick_f32_geom(tpw, lean) : exact ? pick_f32_exact(tpw, lean) : pick_f32_lean(tpw, lean);
 }
@@ -327,9 +327,9 @@ size_t batched_smem(const phast_ctx* c, bool fp32, int wpc, SlotLayout* L) {
 }
 
 // Shared memory of a one-walker-per-thread tile of wpc walkers (wpc / 32 warp slots).
-size_t lane_smem(const phast_ctx* c, bool fp32, int wpc, LaneLayout* L) {
-    *L = fp32 ? lane_layout<float>(c->max_N, c->max_nc, c->max_chain)
-              : lane_layout<double>(c->max_N, c->max_nc, c->max_chain);
+size_t lane_smem(const phast_ctx* c, bool fp32, int wpc, LaneLayout* L, bool shared_trials = false) {
+    *L = fp32 ? lane_layout<float>(c->max_N, c->max_nc, c->max_chain, shared_trials)
+              : lane_layout<double>(c->max_N, c->max_nc, c->max_chain, shared_trials);
     return sizeof(SysDesc) + (size_t)align16(4 * c->max_bins) + (size_t)(wpc / 32) * L->bytes;
 }
 
@@ -380,6 +380,23 @@ int fill_args(const phast_ctx* c, int64_t n_sweeps, const double* lnW, int n_jk,
     // the walkers of a tile add at most wpc n_sweeps N counts to its shared histogram
     a->hist_flush_on = (uint64_t)wpc * (uint64_t)n_sweeps * (uint64_t)c->max_N >= (uint64_t)c->hist_flush;
     return PHAST_OK;
+}
+
+// One-walker-per-thread tiles: the number that their count is rounded up to.  A warp takes the
+// union of its walkers' paths and each SM has four schedulers, so up to four warps per SM cost
+// little more than one, and beyond that every further warp costs its own time: the walkers go to
+// four warps per SM if these hold them, else to as few as hold them, the same number on each SM.
+// 13-mers in a sphere, 1 x 32 tiles, 4 sweeps, all resident CTAs -> this rule: 4096 walkers
+// 5.5 -> 4.8 ms, 16,384 walkers 7.8 -> 6.0 ms; one warp per SM takes 4.2 ms for 1000 walkers,
+// four take 2.9.
+int lane_round(const phast_ctx* c, int wpc, int per_sm, int n_sm) {
+    int64_t walkers = 0, tiles = 0;
+    for (int s = 0; s < c->n_sys; ++s) {
+        walkers += c->desc[s].n_walkers;
+        tiles += (c->desc[s].n_walkers + wpc - 1) / wpc;
+    }
+    if (walkers <= 128ll * n_sm) return n_sm * std::min(per_sm, std::max(1, 128 / wpc));
+    return tiles <= (int64_t)per_sm * n_sm ? n_sm : per_sm * n_sm;
 }
 
 // Tiles of at most wpc walkers, as many as make whole rounds of the grid: the
@@ -486,9 +503,29 @@ int prepare_batched(phast_ctx* c, const SweepArgs& a0, int tpw, int wpc, bool fp
         }
     }
     PHAST_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
+    if (tpw == 1 && fp32) {
+        // trial records in shared memory, if that leaves room for as many CTAs, or for all there is
+        // work for (13-mers in a sphere, 4 sweeps: 4096 walkers in 1 x 32 tiles 6.1 -> 5.5 ms, 65,536
+        // in 1 x 128 tiles 17.7 -> 16.7); fewer resident warps would cost more than the records in L2
+        LaneLayout with;
+        const size_t sm = lane_smem(c, fp32, wpc, &with, true);
+        const batched_fn fn = pick_lane(true, uses_geometry(c), true);
+        int n_tiles = 0, per_sm_with = 0;
+        for (int s = 0; s < c->n_sys; ++s) n_tiles += (c->desc[s].n_walkers + wpc - 1) / wpc;
+        if (sm + 64 <= (size_t)max_sm) {
+            PHAST_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            PHAST_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_with, fn, L->threads, sm));
+        }
+        if (per_sm_with >= per_sm || (per_sm_with >= 1 && per_sm_with * n_sm >= n_tiles)) {
+            L->fn = fn;
+            L->smem = sm;
+            L->a.LL = with;
+            per_sm = per_sm_with;
+        }
+    }
     if (per_sm < 1) return phast_set_error(PHAST_EINVAL, "tile of %d x %d does not fit on an SM", tpw, wpc);
     L->grid = per_sm * n_sm;
-    layout_tiles(c, wpc, L->grid, &L->a);
+    layout_tiles(c, wpc, tpw == 1 ? lane_round(c, wpc, per_sm, n_sm) : L->grid, &L->a);
     if (L->grid > L->a.n_tiles) L->grid = L->a.n_tiles;
     return PHAST_OK;
 }

@@ -45,7 +45,13 @@ batched_fn pick_f32_lean(int tpw, bool lean);     // FP32, no geometry
 batched_fn pick_f32_exact(int tpw, bool lean);    // and the exact path of the torsion terms
 batched_fn pick_f32_geom(int tpw, bool lean);     // the paper's geometry
 batched_fn pick_f64(int tpw, bool geom);
-batched_fn pick_lane(bool fp32, bool geom);       // one walker per thread
+batched_fn pick_lane(bool fp32, bool geom, bool shared_trials);   // one walker per thread
+
+// Moves from move index t to the next multiple of period (0: none), at most 2^30.
+__device__ __forceinline__ uint32_t moves_to_period(uint64_t t, uint64_t period) {
+    const uint64_t n = period ? period - t % period : 1ull << 30;
+    return (uint32_t)(n < (1ull << 30) ? n : 1ull << 30);
+}
 
 #ifdef PHAST_SWEEP_KERNELS
 #include "lane.cuh"   // the one-walker-per-thread form (uses SweepArgs)
@@ -99,12 +105,6 @@ __device__ __forceinline__ void recompute_energy(const SysDesc& sd, const double
     g.sync();
     build_working<TPW, PT>(sd, x64, slot, g);
 }
-// Moves from move index t to the next multiple of period (0: none), at most 2^30.
-__device__ __forceinline__ uint32_t moves_to_period(uint64_t t, uint64_t period) {
-    const uint64_t n = period ? period - t % period : 1ull << 30;
-    return (uint32_t)(n < (1ull << 30) ? n : 1ull << 30);
-}
-
 // GEOM: the system types use the paper's own geometry (FENE bonds, container,
 // bond-length or cap moves); without it those branches are compiled out, which
 // keeps the per-move loop short in the instruction cache.
@@ -341,7 +341,7 @@ sweep_batched_kernel(const SweepArgs a) {
 // the CTA's blockDim.x walkers, each warp's walkers in one lane-interleaved
 // shared-memory slot.
 
-template <typename PT, bool GEOM>
+template <typename PT, bool GEOM, bool SH>
 __global__ void __launch_bounds__(kLaneMaxThreads)
 sweep_lane_kernel(const SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -349,7 +349,7 @@ sweep_lane_kernel(const SweepArgs a) {
     SysDesc& sd = *reinterpret_cast<SysDesc*>(smem);
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem + sizeof(SysDesc));
     unsigned char* warps = smem + sizeof(SysDesc) + align16(4 * a.hist_bins);
-    const LaneSlot<PT> slot(warps + (size_t)(threadIdx.x >> 5) * a.LL.bytes, a.LL, threadIdx.x & 31);
+    const LaneSlot<PT, SH> slot(warps + (size_t)(threadIdx.x >> 5) * a.LL.bytes, a.LL, threadIdx.x & 31);
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(a.tile_counter, 1);
         __syncthreads();
@@ -364,7 +364,9 @@ sweep_lane_kernel(const SweepArgs a) {
         const int k = tile - a.tile_start[pos], nt = a.tiles[pos];
         const int W = sd.n_walkers;
         const int w_a = (int)((int64_t)k * W / nt), w_b = (int)((int64_t)(k + 1) * W / nt);
-        const int w_local = w_a + (int)threadIdx.x;
+        const int n_warps = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int per = (w_b - w_a + n_warps - 1) / n_warps;
+        const int w_local = lane < per ? w_a + warp * per + lane : w_b;
         const int blk = jk_block(w_a, W, a.n_jk);
         __syncthreads();
         unsigned long long* hs_tile = a.hist_sum ? a.hist_sum + a.hs_off[s_id] + (int64_t)blk * sd.n_bins : nullptr;
@@ -372,7 +374,7 @@ sweep_lane_kernel(const SweepArgs a) {
             const int mine = jk_block(w_local, W, a.n_jk);
             unsigned long long* hg =
                 (a.hist_sum && mine != blk) ? a.hist_sum + a.hs_off[s_id] + (int64_t)mine * sd.n_bins : nullptr;
-            run_walker_lane<PT, GEOM>(sd, a, s_id, w_local, slot, hist, hs_tile, hg);
+            run_walker_lane<PT, GEOM, SH>(sd, a, s_id, w_local, slot, hist, hs_tile, hg);
         }
         __syncthreads();
         if (hs_tile) {

@@ -2,7 +2,8 @@
 #define PHAST_SWEEP_KERNELS
 #include "sweep_kernels.cuh"
 
-batched_fn pick_lane(bool fp32, bool geom) {
-    return geom ? (fp32 ? sweep_lane_kernel<float, true> : sweep_lane_kernel<double, true>)
-                : (fp32 ? sweep_lane_kernel<float, false> : sweep_lane_kernel<double, false>);
+batched_fn pick_lane(bool fp32, bool geom, bool shared_trials) {
+    if (!fp32) return geom ? sweep_lane_kernel<double, true, false> : sweep_lane_kernel<double, false, false>;
+    if (shared_trials) return geom ? sweep_lane_kernel<float, true, true> : sweep_lane_kernel<float, false, true>;
+    return geom ? sweep_lane_kernel<float, true, false> : sweep_lane_kernel<float, false, false>;
 }
