@@ -458,10 +458,7 @@ __device__ __forceinline__ bool bond_step(const Pos& pos, int o, int n, int l, d
 
 // Steric container (hard wall about the origin): true if (x^2 + y^2) + z^2 <= R^2.
 __device__ __forceinline__ bool inside64(const SysDesc& d, double3 x) {
-    // non-negative values order as their bit patterns, a NaN (either sign) above all
-    const double r2 = xadd(xadd(xmul(x.x, x.x), xmul(x.y, x.y)), xmul(x.z, x.z));
-    return !d.has_sphere ||
-           (__double_as_longlong(r2) & 0x7fffffffffffffffll) <= __double_as_longlong(d.sphere_R2);
+    return !(d.sphere_R2 > 0.0) || xadd(xadd(xmul(x.x, x.x), xmul(x.y, x.y)), xmul(x.z, x.z)) <= d.sphere_R2;
 }
 
 // Lennard-Jones pair of Eq. 2/3 without its coupling: r^-12 - C r^-6 (FP64).

@@ -68,11 +68,11 @@ __device__ __forceinline__ DF df_of(double x) {
     const float h = (float)x;
     return DF{h, (float)(x - (double)h)};
 }
-// Tree sum of the group's DF values; every lane receives lane 0's total.
-template <int TPW>
+// Tree sum of the DF values of the group's first ORD lanes; every lane receives the total.
+template <int TPW, int ORD = TPW>
 __device__ __forceinline__ DF group_sum_df(DF v, const Group<TPW>& g) {
 #pragma unroll
-    for (int o = TPW / 2; o > 0; o >>= 1)
+    for (int o = ORD / 2; o > 0; o >>= 1)
         v = df_add(v, DF{__shfl_down_sync(g.mask, v.hi, o, TPW), __shfl_down_sync(g.mask, v.lo, o, TPW)});
     return DF{__shfl_sync(g.mask, v.hi, 0, TPW), __shfl_sync(g.mask, v.lo, 0, TPW)};
 }
@@ -111,18 +111,17 @@ __host__ __device__ inline SlotLayout slot_layout(int N, int nc, int mc) {
 
 // Per-warp shared-memory layout of the one-walker-per-thread sweep (bytes).
 struct LaneLayout {
-    int r_off, w_off, org_off, newr_off, bytes;
+    int r_off, w_off, org_off, bytes;   // the trial records first
 };
 // shared_trials: the trial records of the moved monomers lie here too (else in the walkers'
 // global scratch).
 template <typename PT>
 __host__ __device__ inline LaneLayout lane_layout(int N, int nc, int mc, bool shared_trials) {
     LaneLayout L;
-    int o = 0;
+    int o = shared_trials ? 32 * (int)sizeof(P4<PT>) * mc : 0;
     L.r_off = o;    o += 32 * (int)sizeof(P4<PT>) * N;
     L.w_off = o;    o += 32 * 16 * nc;
     L.org_off = o;  o += 32 * 16 * nc;
-    L.newr_off = o; o += shared_trials ? 32 * (int)sizeof(P4<PT>) * mc : 0;
     L.bytes = o;
     return L;
 }
@@ -259,10 +258,10 @@ __device__ __forceinline__ bool disc_test(uint4 r, float* v1f, float* v2f, float
 // same axis in FP32 mode (whose exact axis is rebuilt at commit from the
 // winning block).  The acceptance words uz, uw are valid on lane 0 only
 // (u = u52(uz, uw) is formed only when the acceptance test needs it).
-template <int TPW, typename PT, bool GEOM = true, bool EXACT = true>
+template <int TPW, typename PT, bool GEOM = true, bool EXACT = true, int ORD = TPW>
 __device__ Proposal propose_group(const SysDesc& d, uint64_t seed, uint64_t t, uint4 blk, const Group<TPW>& g) {
     // blk: this lane's stream block (block index = lane) of move t
-    constexpr bool SECOND = TPW == 32 && !EXACT;
+    constexpr bool SECOND = ORD == 32 && !EXACT;
     constexpr bool OUT = TPW < 32 || EXACT;   // the Philox rounds out of line
     Proposal P;
     P.angle = 0.0;
@@ -575,7 +574,7 @@ __device__ __forceinline__ void sincos32(float a, float* s, float* c) {
 // (commit_move).  Returns false for a degenerate crankshaft axis or bond step.
 // *jac (bond-length moves, when given): the Hastings factor ((r + delta) / r)^2,
 // exact in FP64 mode, from the FP32 bond length in FP32 mode.
-template <int TPW, typename PT, bool GEOM = true>
+template <int TPW, typename PT, bool GEOM = true, int ORD = TPW>
 __device__ bool make_new_positions(const SysDesc& d, const double* x64, const Proposal& P, const MoveSet& M,
                                    Slot<PT>& s, const Group<TPW>& g, double* jac = nullptr) {
     const int m = M.hi - M.lo + 1;
@@ -633,12 +632,13 @@ __device__ bool make_new_positions(const SysDesc& d, const double* x64, const Pr
                 cx = p.x; cy = p.y; cz = p.z;
             } else if (P.type == PHAST_ROT) {
                 cx = cy = cz = 0.0f;
-                for (int j = o + g.lane; j < o + n; j += TPW) {
+                // every ORD lanes of a wide group form the same sum
+                for (int j = o + (g.lane & (ORD - 1)); j < o + n; j += ORD) {
                     const P4<PT> p = s.r[j];
                     cx += p.x; cy += p.y; cz += p.z;
                 }
 #pragma unroll
-                for (int w = TPW / 2; w > 0; w >>= 1) {
+                for (int w = ORD / 2; w > 0; w >>= 1) {
                     cx += __shfl_xor_sync(g.mask, cx, w, TPW);
                     cy += __shfl_xor_sync(g.mask, cy, w, TPW);
                     cz += __shfl_xor_sync(g.mask, cz, w, TPW);
@@ -1053,7 +1053,7 @@ __device__ __noinline__ PT bond_item(const SysDesc& d, bool fene, P4<PT> a, P4<P
 // and *near is set where one of them lies in the band of fene_w.  tors: likewise the
 // torsion terms go to *tors, and *tnear is set where a dihedral lies in the band of
 // torsion_w.
-template <int TPW, bool GEOM = true, bool EXACT = true>
+template <int TPW, bool GEOM = true, bool EXACT = true, int ORD = TPW>
 __device__ float local_delta32(const SysDesc& d, const Proposal& P, const MoveSet& M, const Slot<float>& s,
                                const Group<TPW>& g, float* fene, bool* near, float* tors, bool* tnear) {
     using PT = float;
@@ -1063,8 +1063,8 @@ __device__ float local_delta32(const SysDesc& d, const Proposal& P, const MoveSe
     if (!GEOM) nf = 0;
     const int nc = GEOM && P.type == PHAST_BOND;   // the stretched bond's pair, counted by the pair loop, taken back
     const int items = 2 * (nb + nt + nf + nc);
-    PT part = (PT)0;
-    for (int it = g.lane; it < items; it += TPW) {
+    // one term of the list: its value with its sign, and which sum it belongs to
+    auto item = [&](int it, PT* v) -> int {
         const bool after = it & 1;
         const int k = it >> 1;
         auto pos = [&](int j) -> P4<PT> {
@@ -1081,19 +1081,67 @@ __device__ float local_delta32(const SysDesc& d, const Proposal& P, const MoveSe
         PT term;
         if (k < nb) term = f.kbend() * bend_w<PT>(pos, o, vb0 + k);
         else if (k < nb + nt) {
-            const PT v = -f.ktors() * torsion_w<PT>(pos, o, jt0 + (k - nb), tnear, EXACT);
-            *tors += after ? v : -v;
-            continue;
+            term = -f.ktors() * torsion_w<PT>(pos, o, jt0 + (k - nb), tnear, EXACT);
+            *v = after ? term : -term;
+            return 1;
         } else {   // a FENE bond or the bond move's pair: out of line (most workloads have neither)
             const bool is_fene = k < nb + nt + nf;
             const int l = o + (is_fene ? fb0 + (k - nb - nt) : P.index);   // the bond's first monomer
             term = bond_item<PT>(d, is_fene, pos(l), pos(l + 1), l, fene ? near : nullptr);
             if (is_fene && fene) {
-                *fene += after ? term : -term;
-                continue;
+                *v = after ? term : -term;
+                return 2;
             }
         }
-        part += after ? term : -term;
+        *v = after ? term : -term;
+        return 0;
+    };
+    PT part = (PT)0;
+    if constexpr (ORD == TPW) {
+        for (int it = g.lane; it < items; it += TPW) {
+            const bool after = it & 1;
+            const int k = it >> 1;
+            auto pos = [&](int j) -> P4<PT> {
+                if (after && j >= M.lo && j <= M.hi) {
+                    const float4* mv = reinterpret_cast<const float4*>(s.newr) + 2 * rec_slot(d, M, j);
+                    const float4 a = mv[0], b = mv[1];
+                    P4<PT> w;
+                    w.x = a.y; w.y = a.w; w.z = b.y; w.tag = __float_as_int(b.z);
+                    return w;
+                }
+                return s.r[j];
+            };
+            const FF<PT> f{d};
+            PT term;
+            if (k < nb) term = f.kbend() * bend_w<PT>(pos, o, vb0 + k);
+            else if (k < nb + nt) {
+                const PT v = -f.ktors() * torsion_w<PT>(pos, o, jt0 + (k - nb), tnear, EXACT);
+                *tors += after ? v : -v;
+                continue;
+            } else {   // a FENE bond or the bond move's pair: out of line (most workloads have neither)
+                const bool is_fene = k < nb + nt + nf;
+                const int l = o + (is_fene ? fb0 + (k - nb - nt) : P.index);   // the bond's first monomer
+                term = bond_item<PT>(d, is_fene, pos(l), pos(l + 1), l, fene ? near : nullptr);
+                if (is_fene && fene) {
+                    *fene += after ? term : -term;
+                    continue;
+                }
+            }
+            part += after ? term : -term;
+        }
+    } else {   // a round's terms by all lanes, added up on the first ORD lanes in their order
+#pragma unroll 1
+        for (int base = 0; base < items; base += TPW) {
+            PT v = (PT)0;
+            const int kind = base + g.lane < items ? item(base + g.lane, &v) : 0;
+            const PT vl = kind == 0 ? v : (PT)0, vt = kind == 1 ? v : (PT)0, vf = GEOM && kind == 2 ? v : (PT)0;
+#pragma unroll
+            for (int h = 0; h < TPW; h += ORD) {
+                part += __shfl_down_sync(g.mask, vl, h, TPW);
+                *tors += __shfl_down_sync(g.mask, vt, h, TPW);
+                if (GEOM) *fene += __shfl_down_sync(g.mask, vf, h, TPW);
+            }
+        }
     }
     return part;
 }
@@ -1141,11 +1189,12 @@ __device__ __forceinline__ PT lj_pair(PT dx, PT dy, PT dz, PT Lj, PT iLj, PT C) 
 // each letter has its own.  Fewer loop bodies keep the one-warp-per-walker builds in the
 // instruction cache (eight 55-mers 108.3 -> 107.0 ms a sweep of 16384 walkers); the
 // sub-warp builds, with one loop in all, lose 2.5 % by the selection.
-template <int RR, bool PBC, bool ONE>
+// parts: the partners' changes one by one; partners beyond the last (t >= U) count 0.
+template <int RR, bool PBC, bool ONE, bool PARTS = false>
 __device__ __forceinline__ float pair_chunk32(const SysDesc& d, const MoveSet& M, int mchain, int m, int t0,
                                               int stride, const P4<float>* __restrict__ r,
                                               const P4<float>* __restrict__ D, const float4* __restrict__ mv,
-                                              int sub = 0, int step = 1) {
+                                              int sub = 0, int step = 1, float* parts = nullptr) {
     // moved monomers i = sub, sub + step, ... of each type segment (step > 1: a
     // partner shared by `step` lanes in the ragged tail)
     const int nc = d.n_chains;
@@ -1154,10 +1203,11 @@ __device__ __forceinline__ float pair_chunk32(const SysDesc& d, const MoveSet& M
 #pragma unroll
     for (int u = 0; u < RR; ++u) {
         const int t = t0 + u * stride;
-        const int j = t < M.lo ? t : t + m;
+        const int jt = t < M.lo ? t : t + m;
+        const int j = PARTS && jt >= d.N ? 0 : jt;
         const P4<float> p = r[j];
         const int cj = p.tag >> 1, tj = p.tag & 1;
-        const bool ex = (j == M.ex0) | (j == M.ex1) | (j == M.ex2);
+        const bool ex = (jt == M.ex0) | (jt == M.ex1) | (jt == M.ex2) | (PARTS && jt >= d.N);
         float qx = p.x, qy = p.y, qz = p.z, Lj = 0.0f, iLj = 0.0f;
         kap[u] = d.kin32;
         if (cj != mchain) {   // into the moved chain's frame
@@ -1230,12 +1280,17 @@ __device__ __forceinline__ float pair_chunk32(const SysDesc& d, const MoveSet& M
     }
     float part = 0.0f;
 #pragma unroll
-    for (int u = 0; u < RR; ++u) part += kap[u] * (acc[u].y - acc[u].x);
+    for (int u = 0; u < RR; ++u) {
+        if constexpr (PARTS) parts[u] = kap[u] * (acc[u].y - acc[u].x);
+        else part += kap[u] * (acc[u].y - acc[u].x);
+    }
     return part;
 }
 
-// This lane's share, summed over its partner chunks in double-float.
-template <int TPW, int R, bool PBC>
+// This lane's share, summed over its partner chunks in double-float.  ORD < TPW (a warp for a
+// tile of ORD lanes per walker): the partners on all lanes, their changes added up on the
+// first ORD lanes in the order that ORD lanes alone would take them in.
+template <int TPW, int R, bool PBC, int ORD = TPW>
 __device__ DF pair_delta32(const SysDesc& d, const MoveSet& M, int mchain, const Slot<float>& s,
                                const Group<TPW>& g) {
     const int m = M.hi - M.lo + 1;
@@ -1244,6 +1299,25 @@ __device__ DF pair_delta32(const SysDesc& d, const MoveSet& M, int mchain, const
     const int full = U / (TPW * R) * (TPW * R);       // partners in chunks of R per lane
     const int full1 = U / TPW * TPW;                    // then one per lane
     DF sum{0.0f, 0.0f};
+    if constexpr (ORD < TPW) {
+        auto add = [&](float v) {
+#pragma unroll
+            for (int h = 0; h < TPW; h += ORD) sum = df_add(sum, DF{__shfl_down_sync(g.mask, v, h, TPW), 0.0f});
+        };
+        int t = g.lane;
+        for (; t - g.lane + TPW < U; t += 2 * TPW) {
+            float v[2];
+            pair_chunk32<2, PBC, true, true>(d, M, mchain, m, t, TPW, s.r, s.D, mv, 0, 1, v);
+            add(v[0]);
+            add(v[1]);
+        }
+        if (t - g.lane < U) {
+            float v = 0.0f;
+            if (t < U) v = pair_chunk32<1, PBC, true>(d, M, mchain, m, t, TPW, s.r, s.D, mv);
+            add(v);
+        }
+        return sum;
+    }
     if constexpr (TPW < 32) {   // small systems: one partner per lane, the shortest code
         for (int t = g.lane; t < U; t += TPW)
             sum = df_add(sum, DF{pair_chunk32<1, PBC, false>(d, M, mchain, m, t, TPW, s.r, s.D, mv), 0.0f});

@@ -42,7 +42,7 @@ struct LaneSlot {
     float4* org;     // [nc][32] chain origins (FP32 values, exact in FP64)
     int lane;
     __device__ __forceinline__ LaneSlot(unsigned char* warp_base, const LaneLayout& L, int lane_)
-        : r((P4<PT>*)(warp_base + L.r_off)), newr(SH ? (P4<PT>*)(warp_base + L.newr_off) : nullptr),
+        : r((P4<PT>*)(warp_base + L.r_off)), newr(SH ? (P4<PT>*)warp_base : nullptr),
           w((float4*)(warp_base + L.w_off)), org((float4*)(warp_base + L.org_off)), lane(lane_) {}
     __device__ __forceinline__ P4<PT>& R(int j) const { return r[j * 32 + lane]; }
     __device__ __forceinline__ P4<PT>& NR(int q) const { return SH ? newr[q * 32 + lane] : newr[q]; }
@@ -264,6 +264,13 @@ __device__ __forceinline__ double lane_pairs64(const SysDesc& d, const MoveSet& 
     return acc;
 }
 
+// inside64, compared as integers: non-negative values order as
+// their bit patterns, a NaN (either sign) above all.
+__device__ __forceinline__ bool inside_wall(const SysDesc& d, double3 x) {
+    const double r2 = xadd(xadd(xmul(x.x, x.x), xmul(x.y, x.y)), xmul(x.z, x.z));
+    return !d.has_sphere || (__double_as_longlong(r2) & 0x7fffffffffffffffll) <= __double_as_longlong(d.sphere_R2);
+}
+
 // Sweeps between re-centrings of the FP32 working copy on the chain centroids.
 constexpr int kLaneRebuildSweeps = 64;
 
@@ -344,11 +351,11 @@ __device__ void run_walker_lane(const SysDesc& sd, const SweepArgs& a, int s_id,
                         const float e = (px * px + py * py + pz * pz) - sd.sphere_R2_32;
                         const float band = 1e-5f * sd.sphere_R2_32;
                         if (e > band) wall = true;
-                        else if (!(e < -band)) wall |= !inside64(sd, y);
+                        else if (!(e < -band)) wall |= !inside_wall(sd, y);
                     }
                 } else {
                     w.x = y.x; w.y = y.y; w.z = y.z;
-                    if (GEOM) wall |= !inside64(sd, y);
+                    if (GEOM) wall |= !inside_wall(sd, y);
                 }
                 w.tag = s.R(M.lo + q).tag;
                 s.NR(q) = w;

@@ -326,6 +326,11 @@ size_t batched_smem(const phast_ctx* c, bool fp32, int wpc, SlotLayout* L) {
     return sizeof(SysDesc) + (size_t)align16(4 * c->max_bins) + (size_t)wpc * L->bytes;
 }
 
+// A warp per walker for tiles of 8 or 16 lanes (prepare_batched).
+batched_fn pick_wide(int tpw, bool geom, bool exact, bool lean) {
+    return geom ? pick_f32_geom_wide(tpw, lean) : exact ? pick_f32_exact_wide(tpw, lean) : pick_f32_lean_wide(tpw, lean);
+}
+
 // Shared memory of a one-walker-per-thread tile of wpc walkers (wpc / 32 warp slots).
 size_t lane_smem(const phast_ctx* c, bool fp32, int wpc, LaneLayout* L, bool shared_trials = false) {
     *L = fp32 ? lane_layout<float>(c->max_N, c->max_nc, c->max_chain, shared_trials)
@@ -503,6 +508,32 @@ int prepare_batched(phast_ctx* c, const SweepArgs& a0, int tpw, int wpc, bool fp
         }
     }
     PHAST_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
+    // A tile of 8 or 16 lanes per walker takes a whole warp each when that still holds all walkers
+    // at once: the walkers of a warp take different moves, one after the other, and a lane of a
+    // narrow group has two to four partners where one of a warp has one.  4 sweeps of 256 walkers
+    // of four 9-mers (16 lanes) 0.71 -> 0.54 ms, of 2000 1.30 -> 0.79; 13-mers (8 lanes) 0.62 ->
+    // 0.46, 0.86 -> 0.59.  Beyond that the 64-register build, with twice the warps, still beats 16
+    // lanes (4000 walkers: 1.68 -> 1.42; 8000 on two rounds of it 2.30 against 2.30) but not 8 (0.98
+    // against 1.02).
+    if (fp32 && (tpw == 8 || tpw == 16)) {
+        const int w = std::min(wpc, kMaxTileThreads / 32);
+        SlotLayout S;
+        const size_t sm = batched_smem(c, fp32, w, &S);   // at most L->smem: w <= wpc
+        for (int lean = 0; lean < (tpw == 16 ? 2 : 1); ++lean) {
+            const batched_fn fn = pick_wide(tpw, uses_geometry(c), c->near_straight, lean);
+            int per_sm_wide = 0;
+            PHAST_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            PHAST_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_wide, fn, 32 * w, sm));
+            if ((int64_t)c->W > (int64_t)per_sm_wide * w * n_sm) continue;
+            L->fn = fn;
+            L->smem = sm;
+            L->a.L = S;
+            L->threads = 32 * w;
+            L->a.wpc = wpc = w;
+            per_sm = per_sm_wide;
+            break;
+        }
+    }
     if (tpw == 1 && fp32) {
         // trial records in shared memory, if that leaves room for as many CTAs, or for all there is
         // work for (13-mers in a sphere, 4 sweeps: 4096 walkers in 1 x 32 tiles 6.1 -> 5.5 ms, 65,536

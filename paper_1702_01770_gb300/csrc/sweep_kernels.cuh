@@ -44,6 +44,11 @@ typedef void (*batched_fn)(const SweepArgs);
 batched_fn pick_f32_lean(int tpw, bool lean);     // FP32, no geometry
 batched_fn pick_f32_exact(int tpw, bool lean);    // and the exact path of the torsion terms
 batched_fn pick_f32_geom(int tpw, bool lean);     // the paper's geometry
+// A warp per walker for tiles of tpw lanes, the sums in those lanes' order (the same results);
+// lean: the 64-register build.
+batched_fn pick_f32_lean_wide(int tpw, bool lean);
+batched_fn pick_f32_exact_wide(int tpw, bool lean);
+batched_fn pick_f32_geom_wide(int tpw, bool lean);
 batched_fn pick_f64(int tpw, bool geom);
 batched_fn pick_lane(bool fp32, bool geom, bool shared_trials);   // one walker per thread
 
@@ -110,7 +115,9 @@ __device__ __forceinline__ void recompute_energy(const SysDesc& sd, const double
 // keeps the per-move loop short in the instruction cache.
 // EXACT: FP32 local terms near their hard edges are taken in FP64 on the exact positions
 // (an out-of-line path); always so with GEOM, and for types that start straight.
-template <int TPW, typename PT, bool GEOM, bool EXACT>
+// ORD: the lanes per walker whose order of summation the FP32 sums take (the tile's; the
+// group may be wider).
+template <int TPW, typename PT, bool GEOM, bool EXACT, int ORD = TPW>
 __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int w_local, Slot<PT>& slot,
                            uint32_t* hist, unsigned long long* const* hist_tile, unsigned long long* hist_g,
                            const Group<TPW>& g) {
@@ -140,7 +147,7 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
 
     build_working<TPW, PT>(sd, x64, slot, g);
     int queued = 0;                                         // accepted moves awaiting their FP64 replay
-    const int qcap = TPW < kQueue ? TPW : kQueue;
+    const int qcap = ORD < kQueue ? ORD : kQueue;
     // Every lane holds the walker's scalar state and takes the same decision
     // from the same broadcast values; lane 0 alone writes histograms and counters.
     double lnw_here = __ldg(lnW + bin);
@@ -148,11 +155,11 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
     constexpr bool OUT = TPW < 32 || EXACT;                 // the Philox rounds out of line
     uint4 blk = stream_block<OUT>(seed, t, (uint32_t)g.lane);   // this lane's block of the current move
     while (t != t_end) {
-        const Proposal P = propose_group<TPW, PT, GEOM, EXACT>(sd, seed, t, blk, g);
+        const Proposal P = propose_group<TPW, PT, GEOM, EXACT, ORD>(sd, seed, t, blk, g);
         if constexpr (!GEOM) __builtin_assume(P.type >= 0 && P.type < PHAST_BOND);   // no bond or cap moves
         const MoveSet M = move_set(sd, P.type, P.chain, P.index);
         double jac = 1.0;   // Hastings factor (bond-length moves)
-        const bool ok = make_new_positions<TPW, PT, GEOM>(sd, x64, P, M, slot, g, &jac);
+        const bool ok = make_new_positions<TPW, PT, GEOM, ORD>(sd, x64, P, M, slot, g, &jac);
         // a trial position beyond the container's wall: infinite energy, not evaluated
         bool wall = false;
         if constexpr (GEOM)
@@ -164,11 +171,11 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
         if constexpr (sizeof(PT) == 4) {   // this lane's share in double-float, the group total on every lane
             DF part{0.0f, 0.0f};
             if (eval) {
-                part = sd.box_L > 0.0 ? pair_delta32<TPW, 3, true>(sd, M, P.chain, slot, g)
-                                      : pair_delta32<TPW, 3, false>(sd, M, P.chain, slot, g);
+                part = sd.box_L > 0.0 ? pair_delta32<TPW, 3, true, ORD>(sd, M, P.chain, slot, g)
+                                      : pair_delta32<TPW, 3, false, ORD>(sd, M, P.chain, slot, g);
                 float fene = 0.0f, tors = 0.0f;
                 bool near = false, tnear = false;
-                part = df_add(part, DF{local_delta32<TPW, GEOM, EXACT>(sd, P, M, slot, g, GEOM ? &fene : nullptr,
+                part = df_add(part, DF{local_delta32<TPW, GEOM, EXACT, ORD>(sd, P, M, slot, g, GEOM ? &fene : nullptr,
                                                                        &near, &tors, &tnear), 0.0f});
                 if constexpr (EXACT) {
                     // a FENE bond near its divergence or a dihedral near degenerate: the
@@ -191,7 +198,7 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
                     part = df_add(part, DF{tors, 0.0f});
                 }
             }
-            dE32 = group_sum_df<TPW>(part, g);
+            dE32 = group_sum_df<TPW, ORD>(part, g);
         } else {
             double part = 0.0;
             if (eval) part = local_delta64<TPW, GEOM>(sd, P, M, slot, g) + pair_delta64<TPW>(sd, M, P.chain, slot, g);
@@ -287,7 +294,7 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
 // MINB: CTAs of kMaxTileThreads per SM the registers must allow.  Small systems
 // run a build held to 64 registers (MINB = 2): their moves are short and
 // latency-bound, and twice the warps per SM hide more of it than the spills cost.
-template <int TPW, typename PT, bool GEOM, bool EXACT = true, int MINB = 1>
+template <int TPW, typename PT, bool GEOM, bool EXACT = true, int MINB = 1, int ORD = TPW>
 __global__ void __launch_bounds__(kMaxTileThreads, MINB)
 sweep_batched_kernel(const SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -325,7 +332,7 @@ sweep_batched_kernel(const SweepArgs a) {
             const int mine = jk_block(w_local, W, a.n_jk);
             unsigned long long* hg =
                 (a.hist_sum && mine != blk) ? a.hist_sum + a.hs_off[s_id] + (int64_t)mine * sd.n_bins : nullptr;
-            run_walker<TPW, PT, GEOM, EXACT>(sd, a, s_id, w_local, slot, hist, &s_hs_tile, hg, g);
+            run_walker<TPW, PT, GEOM, EXACT, ORD>(sd, a, s_id, w_local, slot, hist, &s_hs_tile, hg, g);
         }
         __syncthreads();
         unsigned long long* hs_tile = s_hs_tile;
@@ -395,6 +402,12 @@ batched_fn pick_batched32(int tpw, bool lean) {
         case 32: return sweep_batched_kernel<32, float, G, X>;
         default: return nullptr;
     }
+}
+
+template <bool G, bool X>
+batched_fn pick_batched32_wide(int tpw, bool lean) {
+    if (tpw == 16) return lean ? sweep_batched_kernel<32, float, G, X, 2, 16> : sweep_batched_kernel<32, float, G, X, 1, 16>;
+    return tpw == 8 && !lean ? sweep_batched_kernel<32, float, G, X, 1, 8> : (batched_fn) nullptr;
 }
 
 template <bool G>
