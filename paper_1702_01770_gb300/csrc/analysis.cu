@@ -446,7 +446,10 @@ int launch_micro(int K, double e_min, double w, const double* lnW, const uint64_
 // same at each of them, since "clearly" is a change of slope over 1e-9 of the slopes where
 // the test's rounding is below 1e-11.  If some triple is not clear, the chain itself runs.
 // The edges, the rise of beta along them, the barrier and f run on all threads.
-// K = 8000, 17 replicates: 230 us (4.6 ms with the chain on one thread).
+// A cluster's CTAs first thin a stretch of the bins each (a bin below its stretch's hull is
+// below the whole one), then one of them the four hulls put together.
+// K = 8000, 17 replicates: 132 us (4.6 ms with the chain on one thread; 240 us with all bins
+// on one CTA and every span in each round; on clusters of 2 and 8 CTAs 192 and 204 us).
 // ---------------------------------------------------------------------------
 
 // E_k = e_min + (k + 1/2) w, each operation rounded separately.
@@ -519,6 +522,46 @@ __device__ int thin_hull(const double* S, int* hull, int nh, int span, int* coun
     return out;
 }
 
+// The visited bins of [k0, k1) in order; every thread receives their number.
+__device__ int visited_bins(const double* S, int k0, int k1, int* hull, int* counts) {
+    int nh = 0;
+    for (int base = k0; base < k1; base += kThreads) {
+        const int k = base + threadIdx.x;
+        const bool in = k < k1 && is_finite64(S[k]);
+        const unsigned b = __ballot_sync(0xffffffffu, in);
+        if ((threadIdx.x & 31) == 0) counts[threadIdx.x >> 5] = __popc(b);
+        __syncthreads();
+        int before = 0, total = 0;
+#pragma unroll
+        for (int q = 0; q < kThreads / 32; ++q) {
+            before += q < (int)(threadIdx.x >> 5) ? counts[q] : 0;
+            total += counts[q];
+        }
+        if (in) hull[nh + before + __popc(b & ((1u << (threadIdx.x & 31)) - 1u))] = k;
+        nh += total;
+        __syncthreads();
+    }
+    return nh;
+}
+
+// Thins the list to its hull: FP32 rounds while they still remove a sixteenth of it, then
+// FP64 ones until none is removed.  A round takes chords of longer and longer spans while
+// they still remove something (8000 noisy bins: 25 passes, 48 with every span in each round).
+__device__ int thin_rounds(const double* S, int* hull, int nh, int* counts, bool* unsure) {
+    bool f64 = false, u;
+    for (;;) {
+        const int n0 = nh;
+        for (int span = 1; span == 1 || span < nh; span *= 4) {
+            const int n = nh;
+            nh = f64 ? thin_hull<true>(S, hull, nh, span, counts, &u) : thin_hull<false>(S, hull, nh, span, counts, &u);
+            if (span == 1) *unsure = u;
+            if (nh == n) break;
+        }
+        if (f64 && nh == n0) return nh;
+        f64 = f64 || nh >= n0 - n0 / 16;
+    }
+}
+
 // x / b rounded correctly from rb = 1 / b (div_count's correction); plain outside the range
 // where the products stay normal.
 __device__ __forceinline__ double quot(double x, double b, double rb, bool safe) {
@@ -539,6 +582,7 @@ maxwell_kernel(int K, double e_min, double w, const double* __restrict__ lnW,
     __shared__ double red[32];
     __shared__ int counts[kThreads / 32];
     __shared__ int s_nh, s_best_q;
+    __shared__ long long s_top;
     __shared__ double s_bc;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
@@ -546,16 +590,48 @@ maxwell_kernel(int K, double e_min, double w, const double* __restrict__ lnW,
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     const double N = (double)n_monomers;
     double* S0 = cluster.map_shared_rank(S, 0);
-    cluster.sync();   // the first CTA's shared memory exists
-    for (int k = rank * kThreads + threadIdx.x; k < K; k += kMaxwellCtas * kThreads) {
+    // each CTA has a stretch of the bins (at their own places in its S)
+    const int share = (K + kMaxwellCtas - 1) / kMaxwellCtas, k0 = min(rank * share, K), k1 = min(k0 + share, K);
+    long long top = PHAST_KEY_LOWEST;
+    for (int k = k0 + threadIdx.x; k < k1; k += kThreads) {
         const double H = rep_hist(hist, n_blocks, K, r, k);
         double s = nan;
         if (H < 0.0) s = -lnW[k];
         else if (H > 0.0) s = -lnW[k] + log(H);
-        S0[k] = s;
+        S[k] = s;
+        if (!is_nan64(s)) top = max(top, order_key(s));
+    }
+    top = block_max_key(top, reinterpret_cast<long long*>(red));
+    if (threadIdx.x == 0) s_top = top;
+    cluster.sync();
+    for (int c = 0; c < kMaxwellCtas; ++c) top = max(top, *cluster.map_shared_rank(&s_top, c));
+    const double mx = key_value(top);
+    for (int k = k0 + threadIdx.x; k < k1; k += kThreads) {   // read back by the same thread
+        double s = S[k];
+        if (!is_nan64(s)) s -= mx;
+        S[k] = s;
+        if (rank > 0) S0[k] = s;
+    }
+    __syncthreads();
+    int nh = 0;
+    bool unsure = !fast_hull;
+    if (beta_c_in <= 0.0 && !unsure) {   // the stretch's own hull: whatever is below it is below the whole one
+        nh = visited_bins(S, k0, k1, hull, counts);
+        bool u;
+        nh = thin_rounds(S, hull, nh, counts, &u);
+        if (threadIdx.x == 0) s_nh = nh;
     }
     cluster.sync();
     const bool want_f = r == 0 && f_out;
+    if (rank == 0 && beta_c_in <= 0.0 && !unsure) {   // the stretches' hulls one after the other
+        for (int c = 1; c < kMaxwellCtas; ++c) {
+            const int n = *cluster.map_shared_rank(&s_nh, c);
+            const int* other = cluster.map_shared_rank(hull, c);
+            for (int q = threadIdx.x; q < n; q += kThreads) hull[nh + q] = other[q];
+            nh += n;
+        }
+    }
+    cluster.sync();   // the first CTA has all that it reads of the others
     if (rank > 0 && !want_f) return;
     auto f_share = [&](double bc) {   // this CTA's share of f (Eq. 7)
         const bool ok = bc > 0.0, safe = ok && quot_safe(bc);
@@ -571,49 +647,9 @@ maxwell_kernel(int K, double e_min, double w, const double* __restrict__ lnW,
         cluster.sync();   // the first CTA's shared memory is read
         return;
     }
-    long long top = PHAST_KEY_LOWEST;
-    for (int k = threadIdx.x; k < K; k += blockDim.x)
-        if (!is_nan64(S[k])) top = max(top, order_key(S[k]));
-    const double mx = key_value(block_max_key(top, reinterpret_cast<long long*>(red)));
-    __syncthreads();
-    for (int k = threadIdx.x; k < K; k += blockDim.x)
-        if (!is_nan64(S[k])) S[k] -= mx;
     if (threadIdx.x == 0) s_best_q = INT_MAX;
     __syncthreads();
-    int nh = 0;
-    bool unsure = !fast_hull;
-    if (beta_c_in <= 0.0 && !unsure) {
-        // the visited bins in order (compaction of all bins), then the rounds
-        for (int base = 0; base < K; base += blockDim.x) {
-            const int k = base + threadIdx.x;
-            const bool in = k < K && is_finite64(S[k]);
-            const unsigned b = __ballot_sync(0xffffffffu, in);
-            if ((threadIdx.x & 31) == 0) counts[threadIdx.x >> 5] = __popc(b);
-            __syncthreads();
-            int before = 0, total = 0;
-#pragma unroll
-            for (int q = 0; q < kThreads / 32; ++q) {
-                before += q < (int)(threadIdx.x >> 5) ? counts[q] : 0;
-                total += counts[q];
-            }
-            if (in) hull[nh + before + __popc(b & ((1u << (threadIdx.x & 31)) - 1u))] = k;
-            nh += total;
-            __syncthreads();
-        }
-        // FP32 rounds while they still remove a sixteenth of the list, then FP64 ones until none is removed
-        for (int n0 = INT_MAX; nh < n0 - n0 / 16;) {
-            n0 = nh;
-            bool u;
-            for (int span = 1; span == 1 || span < nh; span *= 4) nh = thin_hull<false>(S, hull, nh, span, counts, &u);
-        }
-        for (;;) {
-            const int n0 = nh;
-            nh = thin_hull<true>(S, hull, nh, 1, counts, &unsure);
-            if (nh == n0) break;
-            bool u;
-            for (int span = 4; span < nh; span *= 4) nh = thin_hull<true>(S, hull, nh, span, counts, &u);
-        }
-    }
+    if (beta_c_in <= 0.0 && !unsure) nh = thin_rounds(S, hull, nh, counts, &unsure);
     if (beta_c_in <= 0.0 && unsure) {   // some triple is nearly collinear: the chain itself
         // the chain test of (k-2, k-1, k): 1 drop, 0 keep, 2 not all three visited
         for (int k = threadIdx.x; k < K; k += blockDim.x) {

@@ -136,3 +136,21 @@ def test_replicates_far_from_the_full_histogram(phast, orc, n_blocks):
     _close(r.cV_T.cpu(), o["cV_T"], 1e-10, 1e-12)
     _close(r.E_T_err.cpu(), orc.jackknife([x["E_T"] for x in reps]), 1e-9, 1e-9)
     _close(r.cV_T_err.cpu(), orc.jackknife([x["cV_T"] for x in reps]), 1e-9, 1e-9)
+
+
+@pytest.mark.parametrize("K,lo,hi", [(1, 0, 1), (2, 0, 2), (5, 0, 5), (9, 3, 4), (515, 0, 129), (2049, 600, 1500), (8001, 2000, 2001),
+                                     (8001, 3990, 8001), (16384, 0, 16384)])
+def test_maxwell_of_visits_in_one_stretch_of_the_bins(phast, orc, K, lo, hi):
+    """The hull is put together from four stretches of the bins: visits confined to one or two of them, one visited bin, as few
+    bins as stretches or fewer, and the largest size, a convex dip with noise each."""
+    rng = np.random.default_rng(K + lo)
+    x = np.linspace(-1.0, 1.0, K)
+    S = 40.0 * (-x * x - 2.0 * np.exp(-((x - x[(lo + hi) // 2]) / 0.2) ** 2)) + 5.0 * x + 0.01 * rng.standard_normal(K)
+    visited = (np.arange(K) >= lo) & (np.arange(K) < hi)
+    lnW, H = -np.where(visited, S, 0.0), visited.astype(np.int64)[None]
+    _, rep, _ = phast.phast_maxwell(_dev(lnW), _dev(H), -0.25 * K, 0.5, 20, fd_half_width=1)
+    Sn = np.where(visited, -lnW, np.nan)
+    _, ro = orc.maxwell(Sn - np.nanmax(Sn), -0.25 * K, 0.5, 20)
+    for q, key in enumerate(("beta_c", "eps_1", "eps_2", "latent", "barrier", "found")):
+        got = rep[0, q].item()
+        assert (np.isnan(got) and np.isnan(ro[key])) or abs(got - ro[key]) <= 1e-12 * max(1.0, abs(ro[key])), (key, got, ro[key])
