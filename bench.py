@@ -33,7 +33,7 @@ N_T = 64
 GEOM_WALKERS = 16384
 GEOM_SWEEPS = 100
 FLOPS_OPEN, FLOPS_PBC = 14, 23          # algorithmic flops of one pair evaluation (open / minimum image)
-LAUNCHES_PER_STEP = 5                   # sweep, 3 analysis kernels, Berg update
+LAUNCHES_PER_STEP = 7                   # sweep, 5 analysis kernels, Berg update
 MOVE_NAMES = ("pivot", "translation", "rotation", "crankshaft", "bond", "cap")
 
 
@@ -196,7 +196,7 @@ def run_reference(args):
 # ----------------------------------------------------------------------------
 # GPU arm
 # ----------------------------------------------------------------------------
-SWEEP_SOURCES = ("common.cuh", "group.cuh", "lane.cuh", "sweep.cu")   # what the sweep kernels are compiled from
+SWEEP_SOURCES = ("common.cuh", "group.cuh", "sweep_kernels.cuh", "sweep_f32_lean.cu")   # what the sweep kernel is compiled from
 
 
 def csrc_digest() -> str:
@@ -522,7 +522,7 @@ def run_ours(args):
     roofline = {"bound": "alu", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
                 "frac": achieved_tf / peak_tf, "traffic": traffic_per_launch(args.walkers),
                 "peak_basis": f"derived: {n_sm} SMs x 128 FP32 lanes x 2 flop x {max_mhz:.0f} MHz (max SM clock)",
-                "kernel": "sweep_batched_kernel<32,float,0,1> (no FENE, sphere, bond or cap moves)",
+                "kernel": "sweep_batched_kernel<32,float,0,0,1,32> (no FENE, sphere, bond or cap moves)",
                 "frac_at_median_clock": (achieved_tf / (n_sm * 256 * clocks["sm_mhz"] * 1e6 / 1e12))
                 if clocks.get("sm_mhz") else None,
                 "timed": ("CUDA events around each captured iteration (histogram clear, the sweep kernel, "

@@ -1,7 +1,7 @@
 // energy.cu -- phast_energy (Eq. 2/3 total energy of a batch of
 // configurations) and phast_delta_energy (energy change of explicit moves).
-// One warp per configuration or move, using the same group machinery as the
-// sweep, so these entry points exercise the sweep's own arithmetic.
+// One warp per configuration or move (FP64 energies of larger systems: four), using the
+// same group machinery as the sweep.
 #include "group.cuh"
 
 namespace {

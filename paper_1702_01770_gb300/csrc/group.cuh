@@ -1353,8 +1353,9 @@ __device__ DF pair_delta32(const SysDesc& d, const MoveSet& M, int mchain, const
 // average) a full warp makes two, where four register partners a lane made twelve rounds
 // of mostly empty lanes.  13 FP64 instructions an evaluation, 16 with an image (26 with
 // rint images and a division).  Together with local_delta64 and the FP32 estimates of the
-// bin and of the exponential: a sweep of eight 13-mers takes 125 us, 417 us before.  The partners left out (move_set) are next to the moved
-// range, so the partners are the monomers outside one block.
+// bin and of the exponential: a sweep of eight 13-mers takes 125 us, 417 us before (79 us with
+// the geometry by lanes).  The partners left out (move_set) are next to the moved range, so the
+// partners are the monomers outside one block.
 template <int TPW>
 __device__ double pair_delta64(const SysDesc& d, const MoveSet& M, int mchain, const Slot<double>& s,
                                const Group<TPW>& g) {

@@ -345,8 +345,8 @@ sweep_batched_kernel(const SweepArgs a) {
 }
 
 // One walker per thread (small systems): the same persistent tiles, a tile being
-// the CTA's blockDim.x walkers, each warp's walkers in one lane-interleaved
-// shared-memory slot.
+// at most the CTA's blockDim.x walkers, spread evenly over its warps, each warp's walkers in
+// one lane-interleaved shared-memory slot.
 
 template <typename PT, bool GEOM, bool SH>
 __global__ void __launch_bounds__(kLaneMaxThreads)
