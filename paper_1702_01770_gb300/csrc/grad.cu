@@ -299,6 +299,7 @@ __device__ __forceinline__ Coef<float> coef32(const SysDesc& d, const Grad32Args
 }
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ bool is_inf32(float a) { return (__float_as_int(a) & 0x7fffffff) == 0x7f800000; }
 
 // x - o rounded to FP32, and the FP64 value of a coordinate.
 __device__ __forceinline__ float rel32(double x, float o) { return f64_to_f32(x - f32_to_f64(o)); }
@@ -503,7 +504,8 @@ __device__ __forceinline__ void finish32(const Grad32Args& a, int b, DF E, DF* g
 #pragma unroll
     for (int q = 0; q < 5; ++q)
         if (lane == q) mine = gp[q];
-    const double v = f32_to_f64(mine.hi) + f32_to_f64(mine.lo);
+    // an infinite sum leaves NaN in lo: hi alone
+    const double v = f32_to_f64(mine.hi) + (is_inf32(mine.hi) ? 0.0 : f32_to_f64(mine.lo));
     if (VJP) {
         acc = __fma_rn(gE, v, acc);
     } else {

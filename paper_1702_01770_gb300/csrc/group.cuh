@@ -1556,12 +1556,12 @@ __device__ double full_energy64(const SysDesc& d, const double* x64, const Group
 }
 
 // Full energy with the Lennard-Jones pairs in FP32 (from the working copy; each lane's row sums
-// added in double-float) and the local terms in FP64 (from x64).
+// added in FP64, which holds what FP32 rows add up to beyond its own range and keeps an infinite
+// row infinite) and the local terms in FP64 (from x64).
 static __device__ double full_energy_working32(const SysDesc& d, const double* x64, const Slot<float>& s, const Group<32>& g) {
     using PT = float;
     double part = local_energy64_warp(d, x64, g.lane, 0, 1);
     const PT L = (PT)d.box_L, iL = (PT)d.inv_L;
-    DF rows{0.0f, 0.0f};
     for (int i = 0; i < d.N; ++i) {
         const P4<PT> a = s.r[i];
         const int ci = a.tag >> 1, si = a.tag & 1;
@@ -1579,8 +1579,7 @@ static __device__ double full_energy_working32(const SysDesc& d, const double* x
             PT e = lj_pair<PT>(dx, dy, dz, Lj, iLj, d.C32[2 * si + (b.tag & 1)]);
             row += (ci == cj ? d.kin32 : d.kout32) * e;
         }
-        rows = df_add(rows, DF{row, 0.0f});
+        part += f32_to_f64(row);
     }
-    part += f32_to_f64(rows.hi) + f32_to_f64(rows.lo);
     return g.sum(part);
 }
