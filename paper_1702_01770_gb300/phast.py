@@ -262,18 +262,31 @@ def _device_params(params: torch.Tensor, xyz: torch.Tensor) -> torch.Tensor:
     return params.to(device=xyz.device, dtype=dtype).contiguous()
 
 
+def _plain_gradient(g: torch.Tensor) -> bool:
+    """Whether an incoming gradient is only its values: not differentiated itself (create_graph), without a
+    forward-mode tangent, and with storage a kernel can read (a batched gradient under vmap has none)."""
+    if (torch.is_grad_enabled() and g.requires_grad) or torch.autograd.forward_ad.unpack_dual(g).tangent is not None:
+        return False
+    try:
+        g.data_ptr()
+    except RuntimeError:
+        return False
+    return True
+
+
 class EnergyFunction(torch.autograd.Function):
     """E(xyz, params) for a batch of conformations of one system; params are the five
     force-field parameters (ff_params order).  The backward pass recomputes the forward
     one in the same kernel (nothing is kept but the inputs).  With FP32 pair terms, FP32 and
     FP64 coordinates are read and their gradients written as they are (scaled by the incoming
-    gradient and, for the parameters, summed in the kernel)."""
+    gradient and, for the parameters, summed in the kernel); an incoming gradient that is
+    itself differentiated or batched scales them as a tensor expression."""
 
     @staticmethod
     def forward(ctx, xyz, params, system, pair_precision):
         # the parameters stay where they are (no copy to the host, no synchronisation)
         ctx.save_for_backward(xyz, params)
-        ctx.system, ctx.pair_precision = system, pair_precision
+        ctx.system, ctx.pair_precision, ctx.structs = system, pair_precision, None
         if pair_precision == 32 and xyz.dtype in _BITS:
             x, p = xyz.contiguous(), _device_params(params, xyz)
             ctx.structs = st = _CallStructs(system)
@@ -290,7 +303,7 @@ class EnergyFunction(torch.autograd.Function):
     def backward(ctx, gE):
         xyz, params = ctx.saved_tensors
         want_xyz, want_par = ctx.needs_input_grad[:2]
-        if ctx.pair_precision == 32 and xyz.dtype in _BITS:
+        if ctx.structs is not None and xyz.dtype in _BITS and _plain_gradient(gE):
             x, p, st = xyz.contiguous(), _device_params(params, xyz), ctx.structs
             gE = gE.to(torch.float64).contiguous()
             B = x.shape[0] if x.numel() else 0
