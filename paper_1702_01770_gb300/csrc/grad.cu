@@ -314,10 +314,15 @@ template <bool VJP>
 __device__ __forceinline__ void put_grad(double* out, float g, double gE, float, float) {
     *out = VJP ? __dmul_rn(gE, f32_to_f64(g)) : f32_to_f64(g);
 }
+// FP32: g gE with gE in two FP32 parts, rounded once; the FP64 product where the parts or the
+// product leave the range in which they are exact (gE of 0, tiny or huge, overflowing gradients).
+static __device__ __noinline__ float scaled_grad64(float g, double gE) { return (float)((double)g * gE); }
 template <bool VJP>
-__device__ __forceinline__ void put_grad(float* out, float g, double, float gh, float gl) {
-    const float p = __fmul_rn(g, gh);   // g gE, gE in two FP32 parts, rounded once
-    *out = __fadd_rn(p, __fmaf_rn(g, gl, __fmaf_rn(g, gh, -p)));
+__device__ __forceinline__ void put_grad(float* out, float g, double gE, float gh, float gl) {
+    const float p = __fmul_rn(g, gh);
+    const float ap = fabsf(p), ag = fabsf(gh);
+    const bool exact = ap > 0x1p-90f && ap < 0x1p126f && ag > 0x1p-90f && ag < 0x1p126f;
+    *out = exact ? __fadd_rn(p, __fmaf_rn(g, gl, __fmaf_rn(g, gh, -p))) : scaled_grad64(g, gE);
 }
 template <typename IN, bool VJP> struct GradOut { typedef double T; };
 template <> struct GradOut<float, true> { typedef float T; };

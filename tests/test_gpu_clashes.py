@@ -51,3 +51,29 @@ def test_energies_of_clashing_monomers(phast, orc, lens):
         assert abs(E[0] - ref[0]) <= 1e-4 * max(1.0, abs(ref[0])) and np.all(E[1:3] == np.inf)
     p = torch.tensor(phast.ff_params(s), dtype=torch.float32, device="cuda")
     assert torch.all(phast.energy(xt.float(), p, s)[1:3] == np.inf)
+
+
+@pytest.mark.parametrize("lens", [[13], [9, 9]], ids=lambda v: "-".join(map(str, v)))
+def test_fp32_gradients_scaled_beyond_the_range(phast, lens):
+    """FP32 leaves whose gradient times dloss/dE overflows, is infinite, underflows or comes of a dloss/dE that FP32 does not
+    hold: the FP64 product rounded to FP32 (1e-5 of the largest, and the spacing of FP32's subnormals)."""
+    s = _system(lens)
+    w = torch.tensor([1.0, 1.0, 1e30, 1e41, 1e-42, -3e38, 0.0, 1e-39, -1e-60], dtype=torch.float64, device="cuda")
+    x = _walks(lens, len(w))
+    x[1, -1] = x[1, 2] + np.array([1e-5, 0.0, 0.0])
+    x[2, -1] = x[2, 2] + np.array([3e-3, 0.0, 0.0])
+    x[8, -1] = x[8, 2] + np.array([3e-3, 0.0, 0.0])
+    y = torch.from_numpy(x).cuda().float().requires_grad_()
+    p = torch.tensor(phast.ff_params(s), dtype=torch.float32, device="cuda")
+    phast.energy(y, p, s).backward(w)
+    gx = phast.phast_energy_grad(s, y.detach().double(), 32)[1]
+    ref = (w.view(-1, 1, 1) * gx).float()
+    got = y.grad
+    assert torch.equal(got.isinf(), ref.isinf()) and torch.equal(got.isnan(), ref.isnan())
+    assert ref[1:4].isinf().any(dim=2).any(dim=1).all() and ref[5].isinf().any() and not ref[[0, 2, 3, 4, 5, 6, 7, 8]].isnan().any()
+    assert torch.equal(got[got.isinf()], ref[ref.isinf()])
+    fin = ref.isfinite()
+    for b in range(len(w)):
+        g, r = got[b][fin[b]].double(), ref[b][fin[b]].double()
+        if r.numel():
+            assert torch.all((g - r).abs() <= 1e-5 * r.abs().max() + 2.0 ** -148), b
