@@ -257,12 +257,12 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
     for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(full, part, o);
     out = __any_sync(full, out);
     if constexpr (W > 1) {
-        if (lane == 0) red[warp] = out ? INFINITY : part;
-        __syncthreads();
+        if (lane == 0) red[warp] = part;
+        out = __syncthreads_or(out);   // whatever the other terms are
         if (threadIdx.x == 0) {
             double E = 0.0;
             for (int q = 0; q < W; ++q) E += red[q];
-            E_out[b] = E;
+            E_out[b] = out ? INFINITY : E;
         }
     } else {
         if (lane == 0) E_out[b] = out ? INFINITY : part;

@@ -62,3 +62,19 @@ def test_pairs_where_the_paths_part(phast, orc, L):
     assert np.all(np.abs(E - ref) <= 1e-11 * np.maximum(1.0, np.abs(ref))), (E, ref)
     x[0, n:] = x[0, :n]
     assert phast.phast_energy(s, torch.from_numpy(x[:1]).cuda()).item() == np.inf
+
+
+@pytest.mark.parametrize("n", [40, 47, 48, 60, 130])
+@pytest.mark.parametrize("bits", [64, 32])
+def test_the_wall_stands_whatever_the_other_terms_are(phast, n, bits):
+    """A monomer beyond the container's wall: +inf, also where the other terms of the configuration are NaN."""
+    rng = np.random.default_rng(2)
+    s = inputs.System("w", np.array([n], np.int32), inputs.random_sequence(n, 0.5, np.random.Generator(np.random.Philox(1))), 0.0,
+                      k_tors=-0.5, sphere_R=60.0)
+    x = np.array([inputs.random_saw(n, 0.9, rng) for _ in range(4)])
+    x[0, n // 2] = np.nan
+    x[1, 3] += 1000.0
+    x[1, n - 3] = np.nan
+    x[2, n - 1] += 1000.0
+    E = phast.phast_energy(s, torch.from_numpy(x).cuda(), bits).cpu().numpy()
+    assert np.all(E[:3] == np.inf) and np.isfinite(E[3])
