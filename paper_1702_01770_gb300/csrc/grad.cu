@@ -216,7 +216,8 @@ energy_grad64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, dou
                     q.y = mimage64_short(d, q.y);
                     q.z = mimage64_short(d, q.z);
                 }
-                const double k = inter ? d.k_lj_inter : d.k_lj_intra, C = cf.c(2 * si + sj);
+                const double k = inter ? d.k_lj_inter : d.k_lj_intra;
+                const double C = cf.c(j > i ? 2 * si + sj : 2 * sj + si);   // the earlier monomer's letter first
                 const double sv = rcp64(dot3(q, q)), s2 = sv * sv, s3 = s2 * sv, ks3 = k * s3;
                 v[0] = __fma_rn(ks3, s3 - C, v[0]);   // k (s^6 - C s^3)
                 const int cls = si == sj ? 3 + si : 5;
@@ -593,7 +594,7 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
                 const int i1 = i0 + 32;
                 const float4 a0 = r[i0], a1 = i1 < N ? r[i1] : make_float4(-1.0e4f, -1.0e4f, -1.0e4f, 0.0f);
                 const int l0 = __float_as_int(a0.w), l1 = __float_as_int(a1.w);
-                const float same0 = cf.c(3 * l0), same1 = cf.c(3 * l1), ab = cf.c(1);
+                const float same0 = cf.c(3 * l0), same1 = cf.c(3 * l1), ab = 0.5f * (cf.c(1) + cf.c(2));   // as from both ends of a pair
                 const float2 ax = make_float2(a0.x, a1.x), ay = make_float2(a0.y, a1.y), az = make_float2(a0.z, a1.z);
                 float2 e = f2(0.0f);
                 int j0 = i0 + 2, j1 = i1 + 2;
@@ -622,7 +623,7 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
                 const float4 a0 = r[0], q0 = r[N - 1];
                 const float dx = a0.x - q0.x, dy = a0.y - q0.y, dz = a0.z - q0.z;
                 const float sv = fast_rcp(dx * dx + dy * dy + dz * dz), s3 = sv * sv * sv;
-                const float C = __float_as_int(a0.w) == __float_as_int(q0.w) ? cf.c(3 * __float_as_int(a0.w)) : cf.c(1);
+                const float C = __float_as_int(a0.w) == __float_as_int(q0.w) ? cf.c(3 * __float_as_int(a0.w)) : 0.5f * (cf.c(1) + cf.c(2));
                 E = df_add(E, DF{kin * (s3 * (s3 - C)), 0.0f});
             }
         } else {
@@ -827,7 +828,7 @@ energy_grad32_kernel(const SysDesc d, const Grad32Args a) {
                 const int i = has ? row0 + li : row0;
                 const float4 p = r[i];
                 const int ti = __float_as_int(p.w), ci = ti >> 1, si = ti & 1;
-                const float CA = cf.c(2 * si), CB = cf.c(2 * si + 1);
+                const float CA = si ? cf.c(1) : cf.c(0), CB = si ? cf.c(3) : cf.c(1);   // one value for AB and BA, as in the energies
                 float2 Gx = f2(0.0f), Gy = f2(0.0f), Gz = f2(0.0f), Ee = f2(0.0f), PA = f2(0.0f), PB = f2(0.0f);
                 for (int c = 0; c < nc; ++c) {
                     const bool in = c == ci;

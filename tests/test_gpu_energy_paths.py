@@ -78,3 +78,34 @@ def test_the_wall_stands_whatever_the_other_terms_are(phast, n, bits):
     x[2, n - 1] += 1000.0
     E = phast.phast_energy(s, torch.from_numpy(x).cuda(), bits).cpu().numpy()
     assert np.all(E[:3] == np.inf) and np.isfinite(E[3])
+
+
+@pytest.mark.parametrize("lens,L", [([13], 0.0), ([60], 0.0), ([33, 20], 0.0), ([9, 9], 14.0)], ids=["13", "60", "33-20", "9-9p"])
+def test_couplings_that_differ_for_ab_and_ba(phast, orc, lens, L):
+    """C_LJ with AB unlike BA (the ABI takes four values): FP64 energies and derivatives give a pair the earlier monomer's letter
+    first, whatever order the pairs come in; the FP32 derivative kernels give one energy with and without gradients."""
+    import dataclasses
+    s = dataclasses.replace(_system(lens, L), C=(1.0, -0.5, 0.7, 0.5))
+    x = random_conformations(s, 4, seed=sum(lens))
+    if L == 0 and len(lens) > 1:
+        x[:, lens[0]:] += np.array([6.0, 0.0, 0.0])
+    m, xt = oracle_model(orc, s), torch.from_numpy(x).cuda()
+    ref = np.array([orc.energy(m, xb) for xb in x])
+    tol = 1e-11 * np.maximum(1.0, np.abs(ref))
+    assert np.all(np.abs(phast.phast_energy(s, xt).cpu().numpy() - ref) <= tol)
+    E, gx, _ = phast.phast_energy_grad(s, xt, 64)
+    assert np.all(np.abs(E.cpu().numpy() - ref) <= tol)
+    h = 1e-5   # the gradient is that of the energy: central differences of step 1e-5, error under h^2 E''' and 1e-11 E / h
+    for j in (0, 5, s.n_total - 1):
+        for k in range(3):
+            d = np.zeros_like(x)
+            d[:, j, k] = h
+            num = np.array([orc.energy(m, a) - orc.energy(m, b) for a, b in zip(x + d, x - d)]) / (2 * h)
+            assert np.all(np.abs(gx[:, j, k].cpu().numpy() - num) <= 1e-4 * np.maximum(1.0, np.abs(num)))
+    E1 = phast.phast_energy_grad(s, xt, 32)[0].cpu().numpy()
+    E0 = phast.phast_energy_grad(s, xt, 32, want_xyz=False, want_ff=False)[0].cpu().numpy()
+    assert np.all(np.abs(E1 - E0) <= 1e-4 * np.maximum(1.0, np.abs(E1)))
+    c = (-0.5 + 0.7) / 2 if len(lens) == 1 else -0.5   # the one value that the FP32 kernels take for AB and BA
+    m32 = oracle_model(orc, dataclasses.replace(s, C=(1.0, c, c, 0.5)))
+    r32 = np.array([orc.energy(m32, xb) for xb in x])
+    assert np.all(np.abs(E1 - r32) <= 1e-4 * np.maximum(1.0, np.abs(r32)))
