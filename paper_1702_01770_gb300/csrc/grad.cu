@@ -279,6 +279,10 @@ energy_grad64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, dou
 // Bending, torsion and FENE terms are evaluated once each; the terms of a round are added to
 // their first, second, ... monomers in turn, so that the lanes of a step touch disjoint ones.
 // ---------------------------------------------------------------------------
+// Left-out pairs get the squared distance kFar2, rows and partners that do not exist the place
+// kFar: 1 / r^6 and the force then underflow to zero exactly, so they add nothing to whatever
+// the real pairs give (pairs at r = 1000 contribute 1e-18 each).
+constexpr float kFar2 = 1.0e16f, kFar = 1.0e8f;
 constexpr int kGrad32Warps = 8;   // warps of a CTA, fewer where their slots exceed the shared memory
 
 struct Grad32Args {
@@ -556,9 +560,9 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
     const float kin = d.kin32;
     const int mid = N / 2;
     double acc = 0.0;
-    if (GRAD && lane == 0) {   // the dummies sit far away (their terms underflow to zero)
-        if (nA & 1) ps[nA] = make_float4(1.0e4f, 1.0e4f, 1.0e4f, __int_as_float(1 << 20));
-        if (nB & 1) ps[pA + nB] = make_float4(1.0e4f, 1.0e4f, 1.0e4f, __int_as_float(1 << 20));
+    if (GRAD && lane == 0) {   // the dummies
+        if (nA & 1) ps[nA] = make_float4(kFar, kFar, kFar, __int_as_float(1 << 20));
+        if (nB & 1) ps[pA + nB] = make_float4(kFar, kFar, kFar, __int_as_float(1 << 20));
     }
     for (int b = blockIdx.x * warps + w; b < a.B; b += gridDim.x * warps) {
         const IN* x = (const IN*)a.xyz + (size_t)b * N * 3;
@@ -592,7 +596,7 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
             // every pair once; s = 1 holds the bonded pairs and that of the two ends
             for (int i0 = lane; i0 < N; i0 += 64) {
                 const int i1 = i0 + 32;
-                const float4 a0 = r[i0], a1 = i1 < N ? r[i1] : make_float4(-1.0e4f, -1.0e4f, -1.0e4f, 0.0f);
+                const float4 a0 = r[i0], a1 = i1 < N ? r[i1] : make_float4(-kFar, -kFar, -kFar, 0.0f);
                 const int l0 = __float_as_int(a0.w), l1 = __float_as_int(a1.w);
                 const float same0 = cf.c(3 * l0), same1 = cf.c(3 * l1), ab = 0.5f * (cf.c(1) + cf.c(2));   // as from both ends of a pair
                 const float2 ax = make_float2(a0.x, a1.x), ay = make_float2(a0.y, a1.y), az = make_float2(a0.z, a1.z);
@@ -608,8 +612,8 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
                     r2 = __ffma2_rn(dy, dy, r2);
                     r2 = __ffma2_rn(dz, dz, r2);
                     if (2 * s == N) {   // the opposite places: each pair comes twice, the first rows take it
-                        if (2 * i0 >= N) r2.x = 1.0e8f;
-                        if (2 * i1 >= N) r2.y = 1.0e8f;
+                        if (2 * i0 >= N) r2.x = kFar2;
+                        if (2 * i1 >= N) r2.y = kFar2;
                     }
                     const float2 sv = make_float2(fast_rcp(r2.x), fast_rcp(r2.y));
                     const float2 s3 = __fmul2_rn(__fmul2_rn(sv, sv), sv);
@@ -617,7 +621,7 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
                                                   __float_as_int(q1.w) == l1 ? -same1 : -ab);
                     e = __ffma2_rn(s3, __fadd2_rn(s3, nC), e);
                 }
-                E = df_add(E, df_add(DF{kin * e.x, 0.0f}, DF{kin * e.y, 0.0f}));
+                E = df_add(E, df_add(DF{kin * e.x, 0.0f}, DF{i1 < N ? kin * e.y : 0.0f, 0.0f}));
             }
             if (lane == 0) {   // the two ends
                 const float4 a0 = r[0], q0 = r[N - 1];
@@ -649,7 +653,7 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
             for (int i0 = lane; i0 < N; i0 += 64) {
                 const int i1 = i0 + 32;
                 const bool has1 = i1 < N;
-                const float4 a0 = r[i0], a1 = has1 ? r[i1] : make_float4(-1.0e4f, -1.0e4f, -1.0e4f, 0.0f);
+                const float4 a0 = r[i0], a1 = has1 ? r[i1] : make_float4(-kFar, -kFar, -kFar, 0.0f);
                 const int s0 = __float_as_int(a0.w) & 1, s1 = __float_as_int(a1.w) & 1;
                 float2 gx0 = f2(0.0f), gy0 = f2(0.0f), gz0 = f2(0.0f), e0 = f2(0.0f);
                 float2 gx1 = f2(0.0f), gy1 = f2(0.0f), gz1 = f2(0.0f), e1 = f2(0.0f);
@@ -675,8 +679,8 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
                             r2 = __ffma2_rn(dy, dy, r2);
                             r2 = __ffma2_rn(dz, dz, r2);
                             // the row itself and its bonded neighbours (index within one of i): far away
-                            if ((unsigned)(j0 - i + 1) <= 2u) r2.x = 1.0e8f;
-                            if ((unsigned)(j1 - i + 1) <= 2u) r2.y = 1.0e8f;
+                            if ((unsigned)(j0 - i + 1) <= 2u) r2.x = kFar2;
+                            if ((unsigned)(j1 - i + 1) <= 2u) r2.y = kFar2;
                             const float2 sv = make_float2(fast_rcp(r2.x), fast_rcp(r2.y));
                             const float2 s2 = __fmul2_rn(sv, sv), s3 = __fmul2_rn(s2, sv);
                             const float2 fr = __fmul2_rn(__fmul2_rn(s2, s2), __ffma2_rn(m2, s3, Cv));
@@ -725,7 +729,7 @@ energy_grad32_kernel(const SysDesc d, const Grad32Args a) {
     double acc = 0.0;
     if (GRAD)
         for (int c = lane; c < nc; c += 32)
-            ps[d.chain_off[c + 1] + c] = make_float4(1.0e4f, 1.0e4f, 1.0e4f, __int_as_float(2 * kDummy));
+            ps[d.chain_off[c + 1] + c] = make_float4(kFar, kFar, kFar, __int_as_float(2 * kDummy));
     for (int b = blockIdx.x * warps + w; b < a.B; b += gridDim.x * warps) {
         const IN* x = (const IN*)a.xyz + (size_t)b * N * 3;
         for (int c = 0; c < nc; ++c) {                // chain centroids in FP32, summed by the warp
@@ -810,7 +814,7 @@ energy_grad32_kernel(const SysDesc d, const Grad32Args a) {
                     // left out: bonded neighbours (s = 1), the second end of opposite places, s + 1 beyond half
                     const bool x0 = (in0 && j0 == i + 1) || (2 * s == N && 2 * i >= N);
                     const bool x1 = 2 * (s + 1) > N || (2 * (s + 1) == N && 2 * i >= N);
-                    r2 = make_float2(x0 ? 1.0e8f : r2.x, x1 ? 1.0e8f : r2.y);
+                    r2 = make_float2(x0 ? kFar2 : r2.x, x1 ? kFar2 : r2.y);
                     const float2 k = make_float2(x0 ? 0.0f : in0 ? d.kin32 : d.kout32, x1 ? 0.0f : in1 ? d.kin32 : d.kout32);
                     const float2 sv = make_float2(fast_rcp(r2.x), fast_rcp(r2.y));
                     const float2 s3 = __fmul2_rn(__fmul2_rn(sv, sv), sv);
@@ -853,8 +857,8 @@ energy_grad32_kernel(const SysDesc d, const Grad32Args a) {
                         float2 r2 = __fmul2_rn(dx, dx);
                         r2 = __ffma2_rn(dy, dy, r2);
                         r2 = __ffma2_rn(dz, dz, r2);
-                        if ((unsigned)((t0 >> 1) - far) <= 2u) r2.x = 1.0e8f;
-                        if ((unsigned)((t1 >> 1) - far) <= 2u) r2.y = 1.0e8f;
+                        if ((unsigned)((t0 >> 1) - far) <= 2u) r2.x = kFar2;
+                        if ((unsigned)((t1 >> 1) - far) <= 2u) r2.y = kFar2;
                         const float2 sv = make_float2(fast_rcp(r2.x), fast_rcp(r2.y));
                         const float2 s2 = __fmul2_rn(sv, sv), s3 = __fmul2_rn(s2, sv);
                         const float2 Cv = make_float2((t0 & 1) ? CB : CA, (t1 & 1) ? CB : CA);
