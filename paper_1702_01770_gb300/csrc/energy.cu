@@ -7,8 +7,17 @@
 namespace {
 
 constexpr int kWarpsPerBlock = 4;
-constexpr int kSplitMinN = 48;   // FP64 energies: systems from here on take far pairs in double-float
+// FP64 energies: systems from here on take far pairs in double-float, four warps each.  It gains from
+// 40 monomers on (4096 configurations, double-float against FP64 throughout on one warp each: 36
+// monomers 117 and 113 us, 40: 124 and 138, 48: 141 and 198, 64: 176 and 365; of 64 configurations
+// 48 monomers take 19 and 46 us); smaller systems keep the plain form.
+constexpr int kSplitMinN = 48;
 constexpr int kSplitWarps = 4;   // warps of such a configuration
+// The far pairs' relative errors (1e-13 at most, independent) may make up one FP64 rounding (2^-53)
+// of the rest of the energy, as sizes of the lanes' sums: root of the far pairs' squares to the rest
+// at most 2^-53 / 1e-13.  A configuration beyond it (nothing near and no bending: conformations blown
+// up, chains that interact from afar) is taken in FP64 throughout.  Eight 55-mers: 1e-5 of it.
+constexpr float kSplitLimit = 1.1e-3f;
 
 // FP32 pairs: one warp per configuration.
 __global__ void __launch_bounds__(32 * kWarpsPerBlock)
@@ -36,10 +45,10 @@ energy32_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
 // An FP64 instruction holds an SMSP's pipe for 64 to 76 cycles, 13 to 16 of them make a pair,
 // and nearly all pairs of a large system are far apart.  SPLIT: a pair further apart than 4
 // (r^-6 below 2.5e-4) is evaluated in double-float arithmetic (two FP32 numbers, about 120
-// FP32 instructions) on coordinates relative to the chains' centroids, whose relative error
-// of some 1e-13 is below 1e-16 of an energy unit a pair; nearer pairs, and those whose image
-// count or magnitude FP32 does not settle, are collected and take the FP64 instructions, a
-// full warp at a time.
+// FP32 instructions) on coordinates relative to a monomer of its chain; its relative error is
+// some 1e-13, which the near pairs and the bends dwarf (kSplitLimit: else the configuration is
+// taken in FP64); nearer pairs, and those whose image count or magnitude FP32 does not settle,
+// are collected and take the FP64 instructions, a full warp at a time.
 // 1024 configurations of eight 55-mers: 1.01 ms (6.12 ms in FP64 throughout); the largest
 // error against extended precision fell from 1.4e-12 to 3.8e-13.
 // ---------------------------------------------------------------------------
@@ -57,6 +66,25 @@ __device__ __forceinline__ double pair_energy64(const SysDesc& d, const double* 
     const double ir2 = rcp64(dx * dx + dy * dy + dz * dz);
     const double ir6 = ir2 * ir2 * ir2;
     return (inter ? d.k_lj_inter : d.k_lj_intra) * (ir6 * (ir6 - d.C[2 * d.seq[i] + d.seq[j]]));
+}
+
+// part plus the pairs first, first + stride, ... of the flat list.
+__device__ __forceinline__ double add_pairs64(double part, const SysDesc& d, const double* x64, int first, int stride) {
+    const int N = d.N, total = N * (N - 1) / 2, dq = stride / N, dt = stride % N;
+    int s = first / N, i = first % N;
+    for (int idx = first; idx < total; idx += stride) {
+        int j = i + s + 1;
+        if (j >= N) j -= N;
+        if (s > 0 || j != i + 1 || d.chain_of[i] != d.chain_of[j]) part += pair_energy64(d, x64, min(i, j), max(i, j));
+        s += dq;
+        i += dt;
+        if (i >= N) { i -= N; ++s; }
+    }
+    return part;
+}
+// A lane's share of a configuration's energy, all of it in FP64.
+static __device__ __noinline__ double whole_energy64(const SysDesc& d, const double* x64, int lane, int w, int W) {
+    return add_pairs64(local_energy64_warp(d, x64, lane, w, W), d, x64, w * 32 + lane, 32 * W);
 }
 
 // a - b and a + b with their rounding errors (TwoSum).
@@ -101,22 +129,23 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ NearPair s_near[W > 1 ? W : kWarpsPerBlock][64];
     __shared__ double red[32];
+    __shared__ float2 s_size[W];   // SPLIT: the warps' sums of far pairs squared, and of the size of the rest
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int w = W > 1 ? warp : 0;                                   // the warp's number within the configuration
     const int b = W > 1 ? blockIdx.x : blockIdx.x * kWarpsPerBlock + warp;
     if (b >= B) return;
     const unsigned full = 0xffffffffu;
-    const int N = d.N, nc = d.n_chains;
+    const int N = d.N;
     const double* x64 = xyz + (size_t)b * N * 3;
     double part = local_energy64_warp(d, x64, lane, w, W);
     bool out = false;   // a monomer beyond the container's wall: infinite energy
     if (d.has_sphere)
         for (int j = w * 32 + lane; j < N; j += 32 * W) out |= !inside64(d, ld3(x64 + 3 * j));
-    const int total = N * (N - 1) / 2;
-    const int dq = 32 * W / N, dt = 32 * W % N;
-    int idx = w * 32 + lane;
-    int s = idx / N, i = idx % N;
     if constexpr (SPLIT) {
+        const int nc = d.n_chains, total = N * (N - 1) / 2;
+        const int dq = 32 * W / N, dt = 32 * W % N;
+        int idx = w * 32 + lane;
+        int s = idx / N, i = idx % N;
         // records: (x, y, z, letter | chain << 1) and the low parts, relative to the chain's centroid;
         // origin differences in two parts; the chain origins themselves
         float4* hi = reinterpret_cast<float4*>(smem);
@@ -124,20 +153,10 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
         float4* Dh = lo + N;
         float4* Dl = Dh + nc * nc;
         double* org = reinterpret_cast<double*>(Dl + nc * nc);
-        for (int c = warp; c < nc; c += W) {   // any point near the chain will do
-            const int o = d.chain_off[c], n = d.chain_off[c + 1] - o;
-            float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-            for (int j = o + lane; j < o + n; j += 32) {
-                sx += f64_to_f32(x64[3 * j]);
-                sy += f64_to_f32(x64[3 * j + 1]);
-                sz += f64_to_f32(x64[3 * j + 2]);
-            }
-            for (int m = 16; m > 0; m >>= 1) {
-                sx += __shfl_xor_sync(full, sx, m);
-                sy += __shfl_xor_sync(full, sy, m);
-                sz += __shfl_xor_sync(full, sz, m);
-            }
-            if (lane < 3) org[3 * c + lane] = f32_to_f64((lane == 0 ? sx : lane == 1 ? sy : sz) / (float)n);
+        // a monomer of the chain, taken whole: x - origin then loses nothing however far out the chain is
+        for (int e = threadIdx.x; e < 3 * nc; e += 32 * W) {
+            const int c = e / 3, o = d.chain_off[c], n = d.chain_off[c + 1] - o;
+            org[e] = x64[3 * (o + n / 2) + (e - 3 * c)];
         }
         __syncthreads();
         auto split = [](double v, float* h, float* l) {
@@ -172,6 +191,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
         for (int q = 0; q < 4; ++q) split(d.C[q], &Ch[q], &Cl[q]);
         __syncthreads();
         DF in{0.0f, 0.0f}, ex{0.0f, 0.0f};   // far pairs within chains and between them
+        float squares = 0.0f;                // sum of their squares
         int n_near = 0;
         NearPair* near = s_near[warp];
         auto drain = [&](int n) {   // the first n of the list
@@ -222,6 +242,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
                         const float wh = __fmul_rn(c3, u);
                         const float wl = __fmaf_rn(c3, ul, __fmaf_rn(c3l, u, __fmaf_rn(c3, u, -wh)));
                         const DF v = df_add(inter ? ex : in, DF{wh, wl});
+                        squares = __fmaf_rn(wh, wh, squares);
                         if (inter) ex = v;
                         else in = v;
                     }
@@ -243,16 +264,26 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
             if (i >= N) { i -= N; ++s; }
         }
         drain(n_near);
-        part += d.k_lj_intra * (f32_to_f64(in.hi) + f32_to_f64(in.lo)) + d.k_lj_inter * (f32_to_f64(ex.hi) + f32_to_f64(ex.lo));
-    } else {
-        for (; idx < total; idx += 32 * W) {
-            int j = i + s + 1;
-            if (j >= N) j -= N;
-            if (s > 0 || j != i + 1 || d.chain_of[i] != d.chain_of[j]) part += pair_energy64(d, x64, min(i, j), max(i, j));
-            s += dq;
-            i += dt;
-            if (i >= N) { i -= N; ++s; }
+        // the far pairs' errors against one rounding of everything else (see kSplitLimit)
+        float rest = fabsf(f64_to_f32(part));
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) {
+            squares += __shfl_xor_sync(full, squares, m);
+            rest += __shfl_xor_sync(full, rest, m);
         }
+        if (lane == 0) s_size[warp] = make_float2(squares, rest);
+        __syncthreads();
+        float2 size = s_size[0];
+#pragma unroll
+        for (int q = 1; q < W; ++q) {
+            size.x += s_size[q].x;
+            size.y += s_size[q].y;
+        }
+        const float k = fmaxf(fabsf(d.kin32), fabsf(d.kout32)), far = k * sqrtf(size.x);
+        if (!(size.y > 1e-12f && far <= kSplitLimit * size.y)) part = whole_energy64(d, x64, lane, w, W);
+        else part += d.k_lj_intra * (f32_to_f64(in.hi) + f32_to_f64(in.lo)) + d.k_lj_inter * (f32_to_f64(ex.hi) + f32_to_f64(ex.lo));
+    } else {
+        part = add_pairs64(part, d, x64, w * 32 + lane, 32 * W);
     }
     for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(full, part, o);
     out = __any_sync(full, out);

@@ -109,3 +109,51 @@ def test_couplings_that_differ_for_ab_and_ba(phast, orc, lens, L):
     m32 = oracle_model(orc, dataclasses.replace(s, C=(1.0, c, c, 0.5)))
     r32 = np.array([orc.energy(m32, xb) for xb in x])
     assert np.all(np.abs(E1 - r32) <= 1e-4 * np.maximum(1.0, np.abs(r32)))
+
+
+EXTENDED = [("walks", [60], 0.0, {}, 0.0, 1.0, 0.0), ("longer walks", [150], 0.0, {}, 0.0, 1.0, 0.0),
+            ("blown up", [60], 0.0, dict(k_bend=0.0), 0.0, 8.0, 0.0), ("blown up far", [60], 0.0, dict(k_bend=0.0), 0.0, 1.0e4, 0.0),
+            ("chains from afar", [60, 60], 0.0, dict(k_bend=0.0, k_lj_intra=0.0), 60.0, 1.0, 0.0),
+            ("chains from afar in a box", [60, 60], 300.0, dict(k_bend=0.0, k_lj_intra=0.0), 60.0, 1.0, 0.0),
+            ("1e9 out", [60], 0.0, {}, 0.0, 1.0, 1.0e9), ("1e12 out", [60], 0.0, {}, 0.0, 1.0, 1.0e12),
+            ("chains 1e12 out", [30, 30], 0.0, {}, 6.0, 1.0, 1.0e12)]
+
+
+def _extended(s, x):
+    """Energy of configurations x in extended precision: bending and Lennard-Jones terms, and the sum of their sizes."""
+    x = x.astype(np.longdouble)
+    off = np.concatenate([[0], np.cumsum(s.chain_len)])
+    chain = np.repeat(np.arange(len(s.chain_len)), s.chain_len)
+    terms = []
+    for c in range(len(s.chain_len)):
+        b = np.diff(x[:, off[c]:off[c + 1]], axis=1)
+        l = np.sqrt((b * b).sum(2))
+        terms.append(np.longdouble(s.k_bend) * (1 - (b[:, 1:] * b[:, :-1]).sum(2) / (l[:, 1:] * l[:, :-1])))
+    i, j = np.triu_indices(s.n_total, 1)
+    keep = ~((chain[i] == chain[j]) & (j == i + 1))
+    i, j = i[keep], j[keep]
+    d, inter = x[:, i] - x[:, j], chain[i] != chain[j]
+    if s.box_L > 0:
+        L = np.longdouble(s.box_L)
+        d = np.where(inter[None, :, None], d - L * np.rint(d / L), d)
+    i6 = 1 / (d * d).sum(2) ** 3
+    k = np.where(inter, np.longdouble(s.k_lj_inter), np.longdouble(s.k_lj_intra))
+    terms.append(k * (i6 * (i6 - np.array(s.C, np.longdouble)[2 * s.seq[i].astype(int) + s.seq[j]])))
+    t = np.concatenate(terms, axis=1)
+    return t.sum(1), np.abs(t).sum(1)
+
+
+@pytest.mark.parametrize("name,lens,L,kw,gap,scale,out", EXTENDED, ids=[e[0].replace(" ", "-") for e in EXTENDED])
+def test_fp64_energies_to_the_last_digits(phast, name, lens, L, kw, gap, scale, out):
+    """Against extended precision: within 16 FP64 roundings of the sum of the terms' sizes (a term has about a dozen, a lane's
+    sum of n / 128 terms and the tree a few more, all of them independent), also where far pairs are all there is and for
+    conformations far from the origin."""
+    s = _system(lens, L, k_tors=0.0)
+    for k, v in kw.items():
+        setattr(s, k, v)
+    rng = np.random.default_rng(1)
+    x = np.array([np.concatenate([inputs.random_saw(n, 0.9, rng) + np.array([gap * i, 0.0, 0.0]) for i, n in enumerate(lens)])
+                  for _ in range(12)]) * scale + out
+    E = phast.phast_energy(s, torch.from_numpy(x).cuda()).cpu().numpy().astype(np.longdouble)
+    ref, size = _extended(s, x)
+    assert np.all(np.abs(E - ref) <= 16 * 2.0 ** -53 * size), ((E - ref) / size / 2.0 ** -53).astype(float)
