@@ -36,19 +36,17 @@ struct Group {
     __device__ __forceinline__ void sync() const { __syncwarp(mask); }
     __device__ __forceinline__ uint32_t bcast(uint32_t v, int src) const { return __shfl_sync(mask, v, src, TPW); }
     __device__ __forceinline__ double bcastd(double v, int src) const { return __shfl_sync(mask, v, src, TPW); }
-    // Tree sum; every lane receives lane 0's total (one value for the whole group).
+    // Tree sum of the first ORD lanes; every lane receives lane 0's total (one value for the whole group).
+    template <int ORD = TPW>
     __device__ __forceinline__ double sum(double v) const {
 #pragma unroll
-        for (int o = TPW / 2; o > 0; o >>= 1) v += __shfl_down_sync(mask, v, o, TPW);
+        for (int o = ORD / 2; o > 0; o >>= 1) v += __shfl_down_sync(mask, v, o, TPW);
         return __shfl_sync(mask, v, 0, TPW);
     }
-    // Tree sum valid on lane 0 only.
-    template <typename T>
-    __device__ __forceinline__ T sum0(T v) const {
-#pragma unroll
-        for (int o = TPW / 2; o > 0; o >>= 1) v += __shfl_down_sync(mask, v, o, TPW);
-        return v;
-    }
+    // The lane's place among the first ORD lanes, beyond every list for the others: sums that are taken
+    // seldom run on these lanes alone, in the order of a group of ORD lanes.
+    template <int ORD>
+    __device__ __forceinline__ int place() const { return ORD < TPW && lane >= ORD ? 1 << 24 : lane; }
 };
 
 // Double-float value hi + lo carried in two FP32 numbers; additions keep each
@@ -743,9 +741,9 @@ __device__ __noinline__ bool container_ok(const SysDesc& d, double* x64, const P
 // torsion_w), summed (+inf for a bond beyond its range, NaN for an exact
 // geometry that is no move).  exact, seed, t and queued as for container_ok:
 // the queued moves are replayed first, so that x64 holds the current
-// coordinates.  The same value on every lane of the group.  Out of line, as
-// container_ok.
-template <int TPW, bool GEOM>
+// coordinates.  The same value on every lane of the group, summed in the order of ORD
+// lanes.  Out of line, as container_ok.
+template <int TPW, bool GEOM, int ORD = TPW>
 __device__ __noinline__ double local_delta_exact(const SysDesc& d, double* x64, const Proposal& P, const MoveSet& M,
                                                  Slot<float>& s, const Group<TPW>& g, bool exact, uint64_t seed,
                                                  uint64_t t, int* queued, bool fene, bool tors) {
@@ -766,7 +764,7 @@ __device__ __noinline__ double local_delta_exact(const SysDesc& d, double* x64, 
     const int nF = fene ? 2 * nf : 0, nT = tors ? 2 * nt : 0;
     double part = 0.0;
     if (ok)
-        for (int k = g.lane; k < nF + nT; k += TPW) {
+        for (int k = g.template place<ORD>(); k < nF + nT; k += ORD) {
             const bool after = k & 1;
             auto pos = [&](int j) -> double3 {
                 const double3 x = ld3(x64 + 3 * j);
@@ -776,7 +774,7 @@ __device__ __noinline__ double local_delta_exact(const SysDesc& d, double* x64, 
                                     : -d.k_tors * torsion_term(pos, o, jt0 + ((k - nF) >> 1));
             part += after ? v : -v;
         }
-    const double dX = g.sum(part);
+    const double dX = g.template sum<ORD>(part);
     return ok ? dX : __longlong_as_double(0x7ff8000000000000ll);
 }
 
@@ -1520,24 +1518,25 @@ static __device__ double local_energy64_warp(const SysDesc& d, const double* x64
 }
 
 // Full FP64 energy (Eq. 2 per chain + inter-chain term of Eq. 3) of the
-// walker at x64; every lane of the group receives the total.
-template <int TPW>
+// walker at x64; every lane of the group receives the total, summed in the order of ORD lanes.
+template <int TPW, int ORD = TPW>
 __device__ double full_energy64(const SysDesc& d, const double* x64, const Group<TPW>& g) {
+    const int first = g.template place<ORD>();
     double part = 0.0;
     auto pos = [&](int j) -> double3 { return ld3(x64 + 3 * j); };
     bool out = false;   // a monomer outside the steric container: infinite energy
     for (int c = 0; c < d.n_chains; ++c) {
         int o = d.chain_off[c], n = d.chain_off[c + 1] - o;
-        for (int k = 1 + g.lane; k <= n - 2; k += TPW) part += d.k_bend * bend_term(pos, o, k);
-        for (int j = g.lane; j <= n - 4; j += TPW) part -= d.k_tors * torsion_term(pos, o, j);
+        for (int k = 1 + first; k <= n - 2; k += ORD) part += d.k_bend * bend_term(pos, o, k);
+        for (int j = first; j <= n - 4; j += ORD) part -= d.k_tors * torsion_term(pos, o, j);
         if (d.k_fene != 0.0)
-            for (int l = g.lane; l <= n - 2; l += TPW) part += fene_term(d, pos, o, l);
+            for (int l = first; l <= n - 2; l += ORD) part += fene_term(d, pos, o, l);
     }
     for (int j = g.lane; j < d.N; j += TPW) out |= !inside64(d, pos(j));
     for (int i = 0; i < d.N; ++i) {
         const double3 xi = pos(i);
         const int ci = d.chain_of[i], si = d.seq[i];
-        for (int j = i + 1 + g.lane; j < d.N; j += TPW) {
+        for (int j = i + 1 + first; j < d.N; j += ORD) {
             const int cj = d.chain_of[j];
             if (ci == cj && j < i + 2) continue;
             const double3 xj = pos(j);
@@ -1551,7 +1550,7 @@ __device__ double full_energy64(const SysDesc& d, const double* x64, const Group
             part += (ci == cj ? d.k_lj_intra : d.k_lj_inter) * e;
         }
     }
-    const double E = g.sum(part);
+    const double E = g.template sum<ORD>(part);
     return __any_sync(g.mask, out) ? INFINITY : E;
 }
 

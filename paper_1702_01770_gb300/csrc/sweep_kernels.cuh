@@ -87,11 +87,11 @@ __host__ __device__ __forceinline__ int jk_block(int w, int W, int n) {
 
 // The FP64 full energy replaces the running one (when in range) and the
 // working copy is rebuilt.
-template <int TPW, typename PT>
+template <int TPW, typename PT, int ORD = TPW>
 __device__ __forceinline__ void recompute_energy(const SysDesc& sd, const double* x64, const double* lnW, Slot<PT>& slot,
                                               const Group<TPW>& g, phast_walker_stats* ls, double& E, int& bin,
                                               double& lnw_here, float& erel) {
-    const double Ef = full_energy64<TPW>(sd, x64, g);
+    const double Ef = full_energy64<TPW, ORD>(sd, x64, g);
     if (g.lane == 0) {
         ls->drift_max = fmax(ls->drift_max, fabs(E - Ef));
         ls->recomputes++;
@@ -115,8 +115,8 @@ __device__ __forceinline__ void recompute_energy(const SysDesc& sd, const double
 // keeps the per-move loop short in the instruction cache.
 // EXACT: FP32 local terms near their hard edges are taken in FP64 on the exact positions
 // (an out-of-line path); always so with GEOM, and for types that start straight.
-// ORD: the lanes per walker whose order of summation the FP32 sums take (the tile's; the
-// group may be wider).
+// ORD: the lanes per walker whose order of summation every sum takes (the tile's; the group may
+// be wider): the walker's results do not depend on how many others share the context.
 template <int TPW, typename PT, bool GEOM, bool EXACT, int ORD = TPW>
 __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int w_local, Slot<PT>& slot,
                            uint32_t* hist, unsigned long long* const* hist_tile, unsigned long long* hist_g,
@@ -183,8 +183,8 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
                     const bool fx = GEOM && (__ballot_sync(g.mask, near) & g.mask);
                     const bool tx = __ballot_sync(g.mask, tnear) & g.mask;
                     if (fx || tx) {
-                        const double dX = local_delta_exact<TPW, GEOM>(sd, x64, P, M, slot, g, false, seed, t,
-                                                                       &queued, fx, tx);
+                        const double dX = local_delta_exact<TPW, GEOM, ORD>(sd, x64, P, M, slot, g, false, seed, t,
+                                                                            &queued, fx, tx);
                         if (g.lane == 0) part = df_add(part, df_of(dX));
                     }
                     if (GEOM && !fx) part = df_add(part, DF{fene, 0.0f});
@@ -270,7 +270,7 @@ __device__ void run_walker(const SysDesc& sd, const SweepArgs& a, int s_id, int 
                     flush_queue<TPW, GEOM>(sd, x64, seed, slot, g, queued);
                     queued = 0;
                 }
-                recompute_energy<TPW, PT>(sd, x64, lnW, slot, g, ls, E, bin, lnw_here, erel);
+                recompute_energy<TPW, PT, ORD>(sd, x64, lnW, slot, g, ls, E, bin, lnw_here, erel);
             }
             left = moves_to_period(t, period);
         }
