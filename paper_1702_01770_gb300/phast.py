@@ -189,6 +189,11 @@ class _Structs:
             self.mp[i].pair_precision = int(pair_precision or 64)
 
 
+def _four(v):
+    """Four coefficients of the ABI (2 s_i + s_j); missing ones are 0."""
+    return v if len(v) == 4 else (*v, *(0.0,) * (4 - len(v)))
+
+
 class _CallStructs:
     """The system and force-field structs of one energy call, packed in one go (the ABI structs of _Structs
     without the multicanonical set-up; the arrays are kept until the call returns)."""
@@ -200,8 +205,8 @@ class _CallStructs:
         self.keep = (cl, sq)
         self.sys = _System.from_buffer_copy(struct.pack("@iPPdd", cl.size, cl.__array_interface__["data"][0],
                                                         sq.__array_interface__["data"][0], s.box_L, s.sphere_R))
-        self.ff = _FF.from_buffer_copy(struct.pack("@15d", s.k_bend, s.k_tors, s.k_lj_intra, s.k_lj_inter, *s.C,
-                                                   s.k_fene, s.fene_r0, s.fene_R, *s.C_F))
+        self.ff = _FF.from_buffer_copy(struct.pack("@15d", s.k_bend, s.k_tors, s.k_lj_intra, s.k_lj_inter, *_four(s.C),
+                                                   s.k_fene, s.fene_r0, s.fene_R, *_four(s.C_F)))
 
 
 def phast_energy(system, xyz: torch.Tensor, pair_precision: int = 64, stream=None) -> torch.Tensor:
