@@ -95,7 +95,7 @@ __host__ __device__ inline SlotLayout slot_layout(int N, int nc, int mc) {
     SlotLayout L;
     int o = 0;
     L.r_off = o;     o = align16(o + (int)sizeof(P4<PT>) * N);
-    L.d_off = o;     o = align16(o + (int)sizeof(P4<PT>) * nc * nc);
+    L.d_off = o;     o = align16(o + (sizeof(PT) == 4 ? (int)sizeof(P4<PT>) * nc * nc : 0));
     L.newr_off = o;  o = align16(o + 32 * mc);   // FP64: P4<double>; FP32: two float4 per moved monomer
     L.orig_off = o;  o = align16(o + 8 * 3 * nc);
     L.geo_off = o;   o = align16(o + 8 * 32);
@@ -176,8 +176,8 @@ __device__ __forceinline__ P4<PT> origin_shift(const SysDesc& d, const double* o
     return q;
 }
 
-// Working copy of a walker: chain origins (FP64 centroid, FP32 mode), relative
-// coordinates, origin-difference table.  x64 is the walker's FP64 [N][3].
+// Working copy of a walker: chain origins (FP64 centroid) and their table of
+// differences (FP32 mode), relative coordinates.  x64 is the walker's FP64 [N][3].
 template <int TPW, typename PT>
 __device__ void build_working(const SysDesc& d, const double* x64, Slot<PT>& s, const Group<TPW>& g) {
     const bool rel = sizeof(PT) == 4;
@@ -203,7 +203,8 @@ __device__ void build_working(const SysDesc& d, const double* x64, Slot<PT>& s, 
         q.tag = (int)d.seq[j] | (c << 1);
         s.r[j] = q;
     }
-    for (int p = g.lane; p < nc * nc; p += TPW) s.D[p] = origin_shift<PT>(d, s.orig, p / nc, p % nc);
+    if constexpr (sizeof(PT) == 4)
+        for (int p = g.lane; p < nc * nc; p += TPW) s.D[p] = origin_shift<PT>(d, s.orig, p / nc, p % nc);
     g.sync();
 }
 
@@ -1097,35 +1098,11 @@ __device__ float local_delta32(const SysDesc& d, const Proposal& P, const MoveSe
     PT part = (PT)0;
     if constexpr (ORD == TPW) {
         for (int it = g.lane; it < items; it += TPW) {
-            const bool after = it & 1;
-            const int k = it >> 1;
-            auto pos = [&](int j) -> P4<PT> {
-                if (after && j >= M.lo && j <= M.hi) {
-                    const float4* mv = reinterpret_cast<const float4*>(s.newr) + 2 * rec_slot(d, M, j);
-                    const float4 a = mv[0], b = mv[1];
-                    P4<PT> w;
-                    w.x = a.y; w.y = a.w; w.z = b.y; w.tag = __float_as_int(b.z);
-                    return w;
-                }
-                return s.r[j];
-            };
-            const FF<PT> f{d};
-            PT term;
-            if (k < nb) term = f.kbend() * bend_w<PT>(pos, o, vb0 + k);
-            else if (k < nb + nt) {
-                const PT v = -f.ktors() * torsion_w<PT>(pos, o, jt0 + (k - nb), tnear, EXACT);
-                *tors += after ? v : -v;
-                continue;
-            } else {   // a FENE bond or the bond move's pair: out of line (most workloads have neither)
-                const bool is_fene = k < nb + nt + nf;
-                const int l = o + (is_fene ? fb0 + (k - nb - nt) : P.index);   // the bond's first monomer
-                term = bond_item<PT>(d, is_fene, pos(l), pos(l + 1), l, fene ? near : nullptr);
-                if (is_fene && fene) {
-                    *fene += after ? term : -term;
-                    continue;
-                }
-            }
-            part += after ? term : -term;
+            PT v;
+            const int kind = item(it, &v);
+            if (kind == 1) *tors += v;
+            else if (GEOM && kind == 2) *fene += v;
+            else part += v;
         }
     } else {   // a round's terms by all lanes, added up on the first ORD lanes in their order
 #pragma unroll 1
@@ -1469,8 +1446,7 @@ __device__ __forceinline__ bool accept_below(double dl, const Proposal& P) {
     return u52(P.uz, P.uw) < exp(dl);
 }
 
-// min(1, W(E')/W(E)): the sign of dlnW by its FP32 image (a negative value that rounds to
-// zero has exp(dlnW) = 1, above every u), then accept_below.
+// min(1, W(E')/W(E)): accepted outright for dlnW >= 0, else by accept_below.
 __device__ __forceinline__ bool accept_weight(double dl, const Proposal& P) {
     return dl >= 0.0 || accept_below(dl, P);
 }
