@@ -498,7 +498,7 @@ __device__ __forceinline__ void chain_terms32(const SysDesc& d, const float4* r,
 // (VJP) this conformation's share of the batch's parameter derivatives, gE dE/dparam, added
 // to acc on lanes 0..4.
 template <bool VJP>
-__device__ __forceinline__ void finish32(const Grad32Args& a, int b, DF E, DF* gp, bool out, double gE, int lane,
+__device__ __forceinline__ void finish32(const Grad32Args& a, unsigned b, DF E, DF* gp, bool out, double gE, int lane,
                                          double& acc, bool want_ff) {
     const unsigned full = 0xffffffffu;
 #pragma unroll
@@ -564,7 +564,7 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
         if (nA & 1) ps[nA] = make_float4(kFar, kFar, kFar, __int_as_float(1 << 20));
         if (nB & 1) ps[pA + nB] = make_float4(kFar, kFar, kFar, __int_as_float(1 << 20));
     }
-    for (int b = blockIdx.x * warps + w; b < a.B; b += gridDim.x * warps) {
+    for (unsigned b = blockIdx.x * warps + w; b < (unsigned)a.B; b += gridDim.x * warps) {   // beyond B it stays below 2^32
         const IN* x = (const IN*)a.xyz + (size_t)b * N * 3;
         // origin: the middle monomer rounded to FP32
         const float ox = as32(x[3 * mid]), oy = as32(x[3 * mid + 1]), oz = as32(x[3 * mid + 2]);
@@ -730,7 +730,7 @@ energy_grad32_kernel(const SysDesc d, const Grad32Args a) {
     if (GRAD)
         for (int c = lane; c < nc; c += 32)
             ps[d.chain_off[c + 1] + c] = make_float4(kFar, kFar, kFar, __int_as_float(2 * kDummy));
-    for (int b = blockIdx.x * warps + w; b < a.B; b += gridDim.x * warps) {
+    for (unsigned b = blockIdx.x * warps + w; b < (unsigned)a.B; b += gridDim.x * warps) {   // beyond B it stays below 2^32
         const IN* x = (const IN*)a.xyz + (size_t)b * N * 3;
         for (int c = 0; c < nc; ++c) {                // chain centroids in FP32, summed by the warp
             const int o = d.chain_off[c], n = d.chain_off[c + 1] - o;
@@ -1042,7 +1042,7 @@ int launch_grad32(const SysDesc& d, grad32_fn fn, bool chain, bool grad, Grad32A
     const size_t sm = sizeof(float4) * (size_t)a.slot_f4 * warps;
     PHAST_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     // a few waves of CTAs, each warp taking several conformations of a large batch
-    int ctas = (a.B + warps - 1) / warps;
+    int ctas = (a.B - 1) / warps + 1;
     *n_ctas = ctas = ctas < kGrad32MaxCtas ? ctas : kGrad32MaxCtas;
     fn<<<ctas, 32 * warps, sm, st>>>(d, a);
     PHAST_CUDA_TRY(cudaGetLastError());
