@@ -320,14 +320,22 @@ __device__ __forceinline__ void put_grad(double* out, float g, double gE, float,
     *out = VJP ? __dmul_rn(gE, f32_to_f64(g)) : f32_to_f64(g);
 }
 // FP32: g gE with gE in two FP32 parts, rounded once; the FP64 product where the parts or the
-// product leave the range in which they are exact (gE of 0, tiny or huge, overflowing gradients).
+// product leave the range in which they are exact (2^-90 to 2^126: gE of 0, tiny or huge, gradients
+// that overflow).
+constexpr unsigned kExactLow = 0x12800000u, kExactSpan = 0x7e800000u - kExactLow;
+__device__ __forceinline__ bool exact_range(float a) { return ((unsigned)__float_as_int(a) & 0x7fffffffu) - kExactLow < kExactSpan; }
 static __device__ __noinline__ float scaled_grad64(float g, double gE) { return (float)((double)g * gE); }
+// gE's parts, 0 outside the range (every product then is too).
+__device__ __forceinline__ void split_gE(double gE, float* gh, float* gl) {
+    const float h = f64_to_f32(gE);
+    const bool in = exact_range(h);
+    *gh = in ? h : 0.0f;
+    *gl = in ? f64_to_f32(gE - f32_to_f64(h)) : 0.0f;
+}
 template <bool VJP>
 __device__ __forceinline__ void put_grad(float* out, float g, double gE, float gh, float gl) {
     const float p = __fmul_rn(g, gh);
-    const float ap = fabsf(p), ag = fabsf(gh);
-    const bool exact = ap > 0x1p-90f && ap < 0x1p126f && ag > 0x1p-90f && ag < 0x1p126f;
-    *out = exact ? __fadd_rn(p, __fmaf_rn(g, gl, __fmaf_rn(g, gh, -p))) : scaled_grad64(g, gE);
+    *out = exact_range(p) ? __fadd_rn(p, __fmaf_rn(g, gl, __fmaf_rn(g, gh, -p))) : scaled_grad64(g, gE);
 }
 template <typename IN, bool VJP> struct GradOut { typedef double T; };
 template <> struct GradOut<float, true> { typedef float T; };
@@ -588,8 +596,7 @@ energy_grad32_chain_kernel(const SysDesc d, const Grad32Args a) {
         float gh = 0.0f, gl = 0.0f;
         if (VJP) {
             gE = a.gE[b];
-            gh = f64_to_f32(gE);
-            gl = f64_to_f32(gE - f32_to_f64(gh));
+            split_gE(gE, &gh, &gl);
         }
         if constexpr (!GRAD) {
             // rows i and i + 32 side by side, each against the partner s places on (cyclically):
@@ -780,8 +787,7 @@ energy_grad32_kernel(const SysDesc d, const Grad32Args a) {
         float gh = 0.0f, gl = 0.0f;
         if (VJP) {
             gE = a.gE[b];
-            gh = f64_to_f32(gE);
-            gl = f64_to_f32(gE - f32_to_f64(gh));
+            split_gE(gE, &gh, &gl);
         }
         if constexpr (!GRAD) {
             // a row against the partners s and s + 1 places on (cyclically), every pair once

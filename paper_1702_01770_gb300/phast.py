@@ -267,10 +267,15 @@ def _device_params(params: torch.Tensor, xyz: torch.Tensor) -> torch.Tensor:
     return params.to(device=xyz.device, dtype=dtype).contiguous()
 
 
+_fwd = torch.autograd.forward_ad
+
+
 def _plain_gradient(g: torch.Tensor) -> bool:
     """Whether an incoming gradient is only its values: not differentiated itself (create_graph), without a
     forward-mode tangent, and with storage a kernel can read (a batched gradient under vmap has none)."""
-    if (torch.is_grad_enabled() and g.requires_grad) or torch.autograd.forward_ad.unpack_dual(g).tangent is not None:
+    if torch.is_grad_enabled() and g.requires_grad:
+        return False
+    if getattr(_fwd, "_current_level", 0) >= 0 and _fwd.unpack_dual(g).tangent is not None:   # only inside a dual level
         return False
     try:
         g.data_ptr()
