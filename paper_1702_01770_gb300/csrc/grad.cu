@@ -348,7 +348,7 @@ __device__ __forceinline__ float bend_vg(const float4& x0, const float4& x1, con
     const float bx = x2.x - x1.x, by = x2.y - x1.y, bz = x2.z - x1.z;
     const float aa = ax * ax + ay * ay + az * az, bb = bx * bx + by * by + bz * bz;
     const float ab = ax * bx + ay * by + az * bz;
-    const float il = rsqrtf(aa * bb);                 // 1 / (|a| |b|)
+    const float il = rsqrtf(aa * bb);                 // 1 / (|a| |b|), for bonds up to 4e9
     const float cs = ab * il;
     const float ia = cs / aa, ib = cs / bb;
     // d cos/d a = b il - cs a / aa, d cos/d b = a il - cs b / bb
@@ -383,18 +383,38 @@ __device__ __noinline__ float torsion_v64(const IN* x64, int j) {
                                0, j);
 }
 
-template <typename IN>
-__device__ __forceinline__ float torsion_vg(const float4& x0, const float4& x1, const float4& x2, const float4& x3,
-                                            float3 g[4], const IN* x64, int j) {
+// The bonds, normals and squared normals of a dihedral in FP32; false where FP32 cannot resolve it
+// (torsion_unresolved32) or hold n11 n22 (the eighth power of a bond length: from 3e4 on).
+struct Dihedral32 {
+    V3<float> u, v, w, n1, n2;
+    float n11, n22;
+};
+__device__ __forceinline__ bool dihedral32(const float4& x0, const float4& x1, const float4& x2, const float4& x3, Dihedral32* D) {
     const V3<float> u{x1.x - x0.x, x1.y - x0.y, x1.z - x0.z}, v{x2.x - x1.x, x2.y - x1.y, x2.z - x1.z},
         w{x3.x - x2.x, x3.y - x2.y, x3.z - x2.z};
     const V3<float> n1 = cross3(u, v), n2 = cross3(v, w);
-    const float n11 = dot3(n1, n1), n22 = dot3(n2, n2);
+    *D = Dihedral32{u, v, w, n1, n2, dot3(n1, n1), dot3(n2, n2)};
     float mx = fmaxf(fmaxf(fabsf(x0.x), fabsf(x0.y)), fabsf(x0.z));
     mx = fmaxf(mx, fmaxf(fmaxf(fabsf(x1.x), fabsf(x1.y)), fabsf(x1.z)));
     mx = fmaxf(mx, fmaxf(fmaxf(fabsf(x2.x), fabsf(x2.y)), fabsf(x2.z)));
     mx = fmaxf(mx, fmaxf(fmaxf(fabsf(x3.x), fabsf(x3.y)), fabsf(x3.z)));
-    if (torsion_unresolved32(n11, n22, mx, true)) return torsion_vg64<IN>(x64, j, g);
+    return !torsion_unresolved32(D->n11, D->n22, mx, true) && fmaxf(D->n11, D->n22) < 1e18f;
+}
+
+template <typename IN>
+__device__ __forceinline__ float torsion_v(const float4& x0, const float4& x1, const float4& x2, const float4& x3, const IN* x64, int j) {
+    Dihedral32 D;
+    if (!dihedral32(x0, x1, x2, x3, &D)) return torsion_v64<IN>(x64, j);
+    return D.n11 * D.n22 < 1e-20f ? 0.0f : dot3(D.n1, D.n2) * rsqrtf(D.n11 * D.n22);
+}
+
+template <typename IN>
+__device__ __forceinline__ float torsion_vg(const float4& x0, const float4& x1, const float4& x2, const float4& x3,
+                                            float3 g[4], const IN* x64, int j) {
+    Dihedral32 D;
+    if (!dihedral32(x0, x1, x2, x3, &D)) return torsion_vg64<IN>(x64, j, g);
+    const V3<float>&u = D.u, &v = D.v, &w = D.w, &n1 = D.n1, &n2 = D.n2;
+    const float n11 = D.n11, n22 = D.n22;
     if (n11 * n22 < 1e-20f) {
         g[0] = g[1] = g[2] = g[3] = make_float3(0.f, 0.f, 0.f);
         return 0.0f;
@@ -456,13 +476,8 @@ __device__ __forceinline__ void chain_terms32(const SysDesc& d, const float4* r,
         float3 g[4];
         if (on) {
             float t;
-            if constexpr (GRAD) {
-                t = torsion_vg<IN>(r[j], r[j + 1], r[j + 2], r[j + 3], g, x64, j);
-            } else {
-                bool nr = false;   // a dihedral FP32 cannot resolve: its FP64 value
-                t = torsion_w<float>(pos, o, base + lane, &nr);
-                if (nr) t = torsion_v64<IN>(x64, j);
-            }
+            if constexpr (GRAD) t = torsion_vg<IN>(r[j], r[j + 1], r[j + 2], r[j + 3], g, x64, j);
+            else t = torsion_v<IN>(r[j], r[j + 1], r[j + 2], r[j + 3], x64, j);
             gp[3] = df_add(gp[3], DF{-t, 0.0f});
             E = df_add(E, DF{-kt * t, 0.0f});
         }

@@ -57,3 +57,15 @@ def test_conformations_blown_up(phast, orc, lens, L, scale):
     rng = np.random.default_rng(1)
     x = np.array([inputs.random_saw(sum(lens), 0.9, rng) for _ in range(4)]) * scale
     _check(phast, orc, s, x)
+
+
+@pytest.mark.parametrize("bond", [1.0e5, 1.0e7])
+@pytest.mark.parametrize("lens,L", [([20], 0.0), ([20], 3.0e9), ([11, 9], 0.0), ([9] * 4, 3.0e9)], ids=["20", "20p", "11-9", "9x4p"])
+def test_local_terms_of_long_bonds(phast, orc, lens, L, bond):
+    """Bending and torsion alone: the products of squares that their FP32 form takes the root of leave FP32 (the eighth power of a
+    bond for the torsion), the terms and gradients do not."""
+    s = _system(lens, L, k_tors=-0.5, k_lj_intra=0.0, k_lj_inter=0.0)
+    rng = np.random.default_rng(1)
+    x = np.array([np.concatenate([inputs.random_saw(n, 0.9, rng) + np.array([12.0 * i, 0.0, 0.0]) for i, n in enumerate(lens)])
+                  for _ in range(4)]) * bond
+    _check(phast, orc, s, x)
