@@ -139,7 +139,8 @@ slopes_kernel(int K, double w, int h, Work wk) {
 // replicates are taken about the full histogram's mean; a replicate whose own mean is more than
 // half its spread from it (the shift would cost its variance digits: at eight spreads an error of
 // 4e-14 of a jackknife error, 7e-16 about its own mean), or whose weights all underflow beside the
-// full histogram's largest, is taken again about its own.
+// full histogram's largest, is taken again about its own; so is the full histogram itself where one
+// bin has all but nothing of the weight and the rounding of its mean would be more than its spread.
 constexpr int kCanonicalThreads = kEntropyThreads;
 constexpr int kCanonicalCtas = 4;
 constexpr int kCanonicalBins = (PHAST_MAX_BINS + kCanonicalCtas - 1) / kCanonicalCtas;
@@ -241,8 +242,8 @@ canonical_kernel(int K, double e_min, double w, const double* __restrict__ lnW, 
             const double Z = m[3 * q], d = m[3 * q + 1] / Z, raw = m[3 * q + 2] / Z;
             double mean = m0 + d, var = raw - d * d;
             // too far from the full histogram's mean, or every weight (nearly) underflowed: the same on every thread
-            if (r > 0 && !(d * d <= 0.25 * var && Z >= 1e-280)) {
-                const double* S = wk.S + (size_t)r * K;
+            if (!(d * d <= 0.25 * var && Z >= 1e-280)) {
+                const double* S = wk.S + (size_t)(r_first + r) * K;
                 double lmax = -INFINITY, z[2] = {0.0, 0.0};
                 auto arg = [&](int k) -> double {
                     const double Ek = bin_energy(e_min, w, k);

@@ -40,3 +40,27 @@ def test_replicates_some_spreads_apart(gap):
         size = np.abs(full[q]) + np.abs(one[q]) + np.abs(two[q]) if q == 0 else np.abs(one[q] - two[q]) / 2
         assert np.all(np.abs(got.cpu().numpy() - full[q]) <= tol * np.abs(full[q]))
         assert np.all(np.abs(err.cpu().numpy() - np.abs(one[q] - two[q]) / 2) <= tol * size)
+
+
+@pytest.mark.parametrize("blocks", [0, 1, 3])
+@pytest.mark.parametrize("binned", [False, True])
+def test_specific_heat_of_a_frozen_system(blocks, binned):
+    """Temperatures so low that one bin has all the weight: c_V is that of the next one, exp(-dE / T) of it (1e-87 to 1e-9), to
+    the rounding of the exponents (2^-53 of 40 / T each) and two dozen others."""
+    from paper_1702_01770_gb300 import phast
+    K, w, e0, n = 500, 0.1, -20.0, 9
+    T = np.array([0.0005, 0.001, 0.002, 0.005])
+    lnW = np.zeros(K)
+    H = None if blocks == 0 else np.full((blocks, K), 7, np.int64)
+    c = lambda a: None if a is None else torch.from_numpy(a).cuda()
+    if binned:
+        r = phast.phast_micro_analysis_binned(c(np.zeros((2, K))), e0, w, c(np.full((2, K), 7, np.int64)), block=1, n_monomers=n, T=c(T))
+    else:
+        r = phast.phast_micro_analysis(c(lnW), e0, w, c(H), n_monomers=n, T=c(T))
+    LD = np.longdouble
+    E = LD(e0) + (np.arange(K).astype(LD) + LD(0.5)) * LD(w)
+    for t, got in zip(T, r.cV_T.cpu().numpy()):
+        p = np.exp(-(E - E[0]) / LD(t))
+        mean = (p * E).sum() / p.sum()
+        ref = (p * (E - mean) ** 2).sum() / p.sum() / (n * LD(t) ** 2)
+        assert abs(got - ref) <= 2.0 ** -53 * (4 * 40 / t + 24) * ref, (t, got, ref)
