@@ -157,3 +157,18 @@ def test_fp64_energies_to_the_last_digits(phast, name, lens, L, kw, gap, scale, 
     E = phast.phast_energy(s, torch.from_numpy(x).cuda()).cpu().numpy().astype(np.longdouble)
     ref, size = _extended(s, x)
     assert np.all(np.abs(E - ref) <= 16 * 2.0 ** -53 * size), ((E - ref) / size / 2.0 ** -53).astype(float)
+
+
+@pytest.mark.parametrize("lens,L", [([5], 0.0), ([33, 20], 0.0), ([9, 9], 14.0)], ids=["5", "33-20", "9-9p"])
+@pytest.mark.parametrize("bits", [64, 32])
+def test_energy_changes_of_configurations_that_have_no_energy(phast, lens, L, bits):
+    """A coordinate that is infinite or NaN: the change of a move elsewhere is NaN."""
+    s = _system(lens, L)
+    x = random_conformations(s, 4, seed=3)
+    if L == 0 and len(lens) > 1:
+        x[:, lens[0]:] += np.array([6.0, 0.0, 0.0])
+    x[1, 0, 1], x[2, 0, 0], x[3, 0, 2] = np.inf, -np.inf, np.nan
+    c = len(lens) - 1
+    move = dict(type=0, chain=c, index=lens[c] - 2, axis=np.array([0.0, 0.6, 0.8]), angle=0.05)
+    dE = phast.phast_delta_energy(s, torch.from_numpy(x).cuda(), [move] * 4, bits).cpu().numpy()
+    assert np.isfinite(dE[0]) and np.all(np.isnan(dE[1:])), dE
