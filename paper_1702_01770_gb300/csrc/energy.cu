@@ -13,10 +13,12 @@ constexpr int kWarpsPerBlock = 4;
 // 48 monomers take 19 and 46 us); smaller systems keep the plain form.
 constexpr int kSplitMinN = 48;
 constexpr int kSplitWarps = 4;   // warps of such a configuration
-// The far pairs' relative errors (1e-13 at most, independent) may make up one FP64 rounding (2^-53)
-// of the rest of the energy, as sizes of the lanes' sums: root of the far pairs' squares to the rest
-// at most 2^-53 / 1e-13.  A configuration beyond it (nothing near and no bending: conformations blown
-// up, chains that interact from afar) is taken in FP64 throughout.  Eight 55-mers: 1e-5 of it.
+// The far pairs' relative errors (independent, at most 1e-13 of their arithmetic and 6e-15 c of their
+// displacements' 48 bits, c the largest coordinate from its chain's origin or difference of origins)
+// may make up one FP64 rounding (2^-53) of the rest of the energy, as sizes of the lanes' sums: root of
+// the far pairs' squares times 1 + 0.06 c to the rest at most 2^-53 / 1e-13.  A configuration beyond it
+// (nothing near and no bending: conformations blown up, chains that interact from afar; unwrapped
+// chains many boxes long) is taken in FP64 throughout.  Eight 55-mers: 1e-5 of it.
 constexpr float kSplitLimit = 1.1e-3f;
 
 // FP32 pairs: one warp per configuration.
@@ -129,7 +131,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ NearPair s_near[W > 1 ? W : kWarpsPerBlock][64];
     __shared__ double red[32];
-    __shared__ float2 s_size[W];   // SPLIT: the warps' sums of far pairs squared, and of the size of the rest
+    __shared__ float4 s_size[W];   // SPLIT: the warps' sums of far pairs squared and of the size of the rest, largest coordinate
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int w = W > 1 ? warp : 0;                                   // the warp's number within the configuration
     const int b = W > 1 ? blockIdx.x : blockIdx.x * kWarpsPerBlock + warp;
@@ -163,6 +165,8 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
             *h = f64_to_f32(v);
             *l = f64_to_f32(v - f32_to_f64(*h));
         };
+        float extent = 0.0f;   // the largest coordinate that a far pair's displacement is made of
+        auto widen = [&](const float4& v) { extent = fmaxf(extent, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fabsf(v.z))); };
         for (int j = threadIdx.x; j < N; j += 32 * W) {
             const int c = d.chain_of[j];
             float4 h, l;
@@ -171,6 +175,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
             split(x64[3 * j + 2] - org[3 * c + 2], &h.z, &l.z);
             h.w = __int_as_float((int)d.seq[j] | (c << 1));
             l.w = 0.0f;
+            widen(h);
             hi[j] = h;
             lo[j] = l;
         }
@@ -180,6 +185,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
             split(mimage64_short(d, org[3 * a] - org[3 * c]), &h.x, &l.x);
             split(mimage64_short(d, org[3 * a + 1] - org[3 * c + 1]), &h.y, &l.y);
             split(mimage64_short(d, org[3 * a + 2] - org[3 * c + 2]), &h.z, &l.z);
+            widen(h);
             Dh[p] = h;
             Dl[p] = l;
         }
@@ -270,16 +276,18 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
         for (int m = 16; m > 0; m >>= 1) {
             squares += __shfl_xor_sync(full, squares, m);
             rest += __shfl_xor_sync(full, rest, m);
+            extent = fmaxf(extent, __shfl_xor_sync(full, extent, m));
         }
-        if (lane == 0) s_size[warp] = make_float2(squares, rest);
+        if (lane == 0) s_size[warp] = make_float4(squares, rest, extent, 0.0f);
         __syncthreads();
-        float2 size = s_size[0];
+        float4 size = s_size[0];
 #pragma unroll
         for (int q = 1; q < W; ++q) {
             size.x += s_size[q].x;
             size.y += s_size[q].y;
+            size.z = fmaxf(size.z, s_size[q].z);
         }
-        const float k = fmaxf(fabsf(d.kin32), fabsf(d.kout32)), far = k * sqrtf(size.x);
+        const float k = fmaxf(fabsf(d.kin32), fabsf(d.kout32)), far = k * sqrtf(size.x) * (1.0f + 0.06f * size.z);
         if (!(size.y > 1e-12f && far <= kSplitLimit * size.y)) part = whole_energy64(d, x64, lane, w, W);
         else part += d.k_lj_intra * (f32_to_f64(in.hi) + f32_to_f64(in.lo)) + d.k_lj_inter * (f32_to_f64(ex.hi) + f32_to_f64(ex.lo));
     } else {

@@ -172,3 +172,22 @@ def test_energy_changes_of_configurations_that_have_no_energy(phast, lens, L, bi
     move = dict(type=0, chain=c, index=lens[c] - 2, axis=np.array([0.0, 0.6, 0.8]), angle=0.05)
     dE = phast.phast_delta_energy(s, torch.from_numpy(x).cuda(), [move] * 4, bits).cpu().numpy()
     assert np.isfinite(dE[0]) and np.all(np.isnan(dE[1:])), dE
+
+
+@pytest.mark.parametrize("bond,L", [(1.0e5, 12.0), (1.0e3, 37.0), (30.0, 12.0)])
+def test_unwrapped_chains_many_boxes_long(phast, bond, L):
+    """Displacements of up to 1e6 between chains come down to half a box by their images: to the rounding of the FP64 coordinates'
+    differences (2 x 2^-53 of the largest in each component, 12 / r of a pair) and 16 roundings of the terms."""
+    s = _system([24, 25, 20], L, k_tors=0.0)
+    rng = np.random.default_rng(1)
+    x = np.array([np.concatenate([inputs.random_saw(n, 0.9, rng) + np.array([0.3, 0.2, 0.4]) * i for i, n in enumerate(s.chain_len)])
+                  for _ in range(12)]) * bond
+    E = phast.phast_energy(s, torch.from_numpy(x).cuda()).cpu().numpy().astype(np.longdouble)
+    ref, size = _extended(s, x)
+    chain = np.repeat(np.arange(3), s.chain_len)
+    i, j = np.triu_indices(s.n_total, 1)
+    i, j = i[chain[i] != chain[j]], j[chain[i] != chain[j]]
+    d = x[:, i] - x[:, j]
+    r = np.sqrt(((d - L * np.rint(d / L)) ** 2).sum(2))
+    steep = (s.k_lj_inter * (12 * r ** -12.0 + 6 * r ** -6.0) / r).sum(1)   # |dE / dr| of the pairs between chains
+    assert np.all(np.abs(E - ref) <= 16 * 2.0 ** -53 * size + 2 * 3 ** 0.5 * 2.0 ** -53 * np.abs(x).max(axis=(1, 2)) * steep)
