@@ -46,7 +46,6 @@ int phast_build_desc(const phast_system* sys, const phast_ff* ff, const phast_mu
         N += n;
         if (n > maxc) maxc = n;
     }
-    for (int c = 0; c < sys->n_chains; ++c) d->inv_len[c] = 1.0 / (double)sys->chain_len[c];
     d->chain_off[sys->n_chains] = N;
     d->n_a_before[0] = 0;
     for (int j = 0; j < N; ++j) d->n_a_before[j + 1] = (uint16_t)(d->n_a_before[j] + (d->seq[j] == 0));

@@ -52,7 +52,6 @@ struct SysDesc {
     float amax32[PHAST_N_MOVES], pad3[2];
     float fene_r0_32, fene_iR32, fene_kR2_32, pad4;
     float C_F32[4];
-    double inv_len[PHAST_MAX_CHAINS];   // 1 / chain length, correctly rounded
     int32_t chain_off[PHAST_MAX_CHAINS + 1];
     int32_t pad1[3];
     uint8_t seq[PHAST_MAX_MONOMERS];
@@ -171,6 +170,16 @@ __device__ __forceinline__ double count_to_f64(int n) {
     const int lz = __clz(n);
     return __hiloint2double(((1053 - lz) << 20) + (int)(((unsigned)n << lz) >> 11), 0);
 }
+// 1 / n of every chain length, correctly rounded (a table of constants, so that the descriptor, which
+// shares a tile's shared memory with its walkers, need not hold them).
+struct InverseCounts {
+    double v[PHAST_MAX_MONOMERS + 1];
+    constexpr InverseCounts() : v{} {
+        for (int n = 1; n <= PHAST_MAX_MONOMERS; ++n) v[n] = 1.0 / n;
+    }
+};
+static __constant__ InverseCounts kInverseCounts = InverseCounts();
+
 // x / n rounded correctly, for a chain length n with rn = 1/n correctly rounded: the
 // quotient x rn and one correction by its exact residual (Markstein's division).  The
 // residual x - n q is exact, and x / n keeps at least 2^-10 of an ulp from the midpoints of
@@ -277,7 +286,7 @@ __device__ __forceinline__ double3 centroid_serial(const SysDesc& d, const doubl
 #pragma unroll
             for (int l = 0; l < w; ++l)
                 if (l + w < n) part[l] = xadd(part[l], part[l + w]);
-        c[k] = div_count(part[0], count_to_f64(n), d.inv_len[ch]);
+        c[k] = div_count(part[0], count_to_f64(n), kInverseCounts.v[n]);
     }
     return make_double3(c[0], c[1], c[2]);
 }

@@ -350,7 +350,7 @@ __device__ __forceinline__ double3 centroid_tree(const SysDesc& d, const At& at,
         return n > 16 ? xadd(p, strided(l + 16, k)) : p;
     };
     auto down = [&](double v, int w) -> double { return n > w ? xadd(v, __shfl_down_sync(g.mask, v, w, TPW)) : v; };
-    const double nd = count_to_f64(n), rn = d.inv_len[c];
+    const double nd = count_to_f64(n), rn = kInverseCounts.v[n];
     if constexpr (TPW == 32) {
         double u = half(g.lane & 15, g.lane >> 4), v = half(g.lane & 15, 2);   // components 0, 1 | 2
         u = down(u, 8);
