@@ -151,8 +151,11 @@ typedef struct phast_ctx phast_ctx;
  * pair_precision 32 or 64 selects the arithmetic of the Lennard-Jones pairs
  * (FP32 positions are taken relative to their chain's FP64 centroid); the
  * bending, torsion and FENE terms and all sums are FP64 (a dihedral of
- * collinear bonds is 0, a decision FP32 coordinates cannot take).  E_out: dev
- * [B].  B = 0 is a no-op. */
+ * collinear bonds is 0, a decision FP32 coordinates cannot take).  64: in
+ * systems of 48 monomers and more, pairs further apart than 4 are evaluated
+ * and summed in double-float (1e-13 of a pair) as long as that stays below an
+ * FP64 rounding of the rest of the energy, else in FP64.  C gives a pair the
+ * earlier monomer's letter first.  E_out: dev [B].  B = 0 is a no-op. */
 int phast_energy(const phast_system* sys, const phast_ff* ff, int32_t B, const double* xyz,
                  int32_t pair_precision, double* E_out, void* stream);
 
@@ -282,8 +285,9 @@ int phast_weight_update(int32_t K, double bin_width, const uint64_t* hist, int32
  * system); grad_ff dev FP64 [B][5] or NULL: dE/d(C_AA, C_BB, C_AB, kappa,
  * kappa_C) -- the Lennard-Jones coefficients of Eq. 1, the torsion weight and
  * the bending weight kappa_C of Eq. 2.  pair_precision 32: FP32 terms on
- * coordinates relative to chain centroids, FP64 sums of the energy and the
- * parameter derivatives; 64: FP64 throughout.  One warp per conformation;
+ * coordinates relative to an origin in each chain, double-float sums of the
+ * energy and the parameter derivatives, one value of C for AB and BA; 64: FP64
+ * throughout.  One warp per conformation;
  * nothing is kept between calls (a backward pass recomputes the forward one).
  * PHAST_EINVAL for bad arguments. */
 int phast_energy_grad(const phast_system* sys, const phast_ff* ff, int32_t B, const double* xyz,

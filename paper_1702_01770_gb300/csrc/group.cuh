@@ -6,12 +6,12 @@
 //     numbers), or plain FP64 copies in the FP64-pair mode;
 //   * the walker's Philox stream drawn by the lanes in parallel (selection
 //     blocks and Marsaglia attempts side by side);
-//   * FP64 move geometry into group scratch; scalar FP64 work (selection,
-//     sin/cos, rotation matrix, bin, acceptance) on one lane only -- FP64 is
-//     the scarce pipe of this chip, so no lane repeats another's FP64 work;
-//   * dE = (bending + torsion window) + (moved x unmoved Lennard-Jones pairs,
-//     R unmoved partners held in registers per lane), in the working
-//     precision, summed per lane and across the group in FP64;
+//   * FP64 move geometry into group scratch, its components spread over the lanes
+//     (an FP64 instruction costs the same on one lane as on all of them); bin and
+//     acceptance by FP32 estimates that settle all but near-ties, on every lane;
+//   * dE = (bending + torsion window) + (moved x unmoved Lennard-Jones pairs): FP32
+//     with unmoved partners held in registers, summed in double-float, or FP64 with the
+//     pairs as one flat list dealt to the lanes;
 //   * full FP64 energies for the drift recompute.
 #pragma once
 
@@ -104,8 +104,6 @@ __host__ __device__ inline SlotLayout slot_layout(int N, int nc, int mc) {
     L.bytes = o;
     return L;
 }
-
-// The one-walker-per-thread form's per-warp layout (lane.cuh).
 
 // Per-warp shared-memory layout of the one-walker-per-thread sweep (bytes).
 struct LaneLayout {
@@ -255,8 +253,8 @@ __device__ __forceinline__ bool disc_test(uint4 r, float* v1f, float* v2f, float
 // only when the first round found no point in the disc.  The winning attempt
 // index is kept; the axis is exact FP64 in FP64 mode and the FP32 image of the
 // same axis in FP32 mode (whose exact axis is rebuilt at commit from the
-// winning block).  The acceptance words uz, uw are valid on lane 0 only
-// (u = u52(uz, uw) is formed only when the acceptance test needs it).
+// winning block).  The acceptance words uz, uw are on every lane (u = u52(uz, uw)
+// is formed only when the acceptance test needs it).
 template <int TPW, typename PT, bool GEOM = true, bool EXACT = true, int ORD = TPW>
 __device__ Proposal propose_group(const SysDesc& d, uint64_t seed, uint64_t t, uint4 blk, const Group<TPW>& g) {
     // blk: this lane's stream block (block index = lane) of move t
