@@ -369,8 +369,8 @@ delta_kernel(const SysDesc d, int B, const double* __restrict__ xyz, const phast
             part += (double)q.hi + (double)q.lo;
         } else {
             part = local_delta64<32>(d, P, M, s, g) + pair_delta64<32>(d, M, P.chain, s, g);
-            bool inf = false;   // an infinite coordinate has no energy to change, as in FP32 mode
-            for (int e = g.lane; e < 3 * d.N; e += 32)
+            bool inf = false;   // an infinite coordinate gives NaN to every pair it is in, as in FP32 mode
+            for (int e = g.lane; M.hi - M.lo + 1 < d.N && e < 3 * d.N; e += 32)
                 inf |= ((unsigned)__double2hiint(x64[e]) & 0x7fffffffu) == 0x7ff00000u && __double2loint(x64[e]) == 0;
             if (inf) part = __longlong_as_double(0x7ff8000000000000ll);
         }

@@ -172,6 +172,9 @@ def test_energy_changes_of_configurations_that_have_no_energy(phast, lens, L, bi
     move = dict(type=0, chain=c, index=lens[c] - 2, axis=np.array([0.0, 0.6, 0.8]), angle=0.05)
     dE = phast.phast_delta_energy(s, torch.from_numpy(x).cuda(), [move] * 4, bits).cpu().numpy()
     assert np.isfinite(dE[0]) and np.all(np.isnan(dE[1:])), dE
+    if len(lens) == 1:   # a rotation of the only chain changes no pair
+        whole = dict(type=2, chain=0, index=0, axis=np.array([0.0, 0.6, 0.8]), angle=0.05)
+        assert np.all(phast.phast_delta_energy(s, torch.from_numpy(x).cuda(), [whole] * 4, bits).cpu().numpy()[:3] == 0.0)
 
 
 @pytest.mark.parametrize("bond,L", [(1.0e5, 12.0), (1.0e3, 37.0), (30.0, 12.0)])
