@@ -565,7 +565,7 @@ __device__ __forceinline__ void finish_part(const Grad32Args& a, double acc, int
 // even length with a far-away dummy), so the coupling C of a run is one value for the row and
 // the parameter sums need no selection; the record carries the partner's index, which excludes
 // the row and its bonded neighbours.  Bound by the FMA pipe of the pair loop (65536
-// conformations of a 55-mer: 137 us forward, 270 us backward; 375 us each, and 170 us of
+// conformations of a 55-mer: 135 us forward, 281 us backward; 375 us each, and 170 us of
 // elementwise passes around them, when both computed everything in FP64 coordinates).
 template <typename IN, bool GRAD, bool VJP>
 __global__ void __launch_bounds__(32 * kGrad32Warps)
