@@ -153,8 +153,8 @@ typedef struct phast_ctx phast_ctx;
  * bending, torsion and FENE terms and all sums are FP64 (a dihedral of
  * collinear bonds is 0, a decision FP32 coordinates cannot take).  64: in
  * systems of 48 monomers and more, pairs further apart than 4 are evaluated
- * and summed in double-float (1e-13 of a pair) as long as that stays below an
- * FP64 rounding of the rest of the energy, else in FP64.  C gives a pair the
+ * and summed in double-float (some 1e-14 of a pair) where that stays below
+ * eight FP64 roundings of the rest of the energy, else in FP64.  C gives a pair the
  * earlier monomer's letter first.  E_out: dev [B].  B = 0 is a no-op. */
 int phast_energy(const phast_system* sys, const phast_ff* ff, int32_t B, const double* xyz,
                  int32_t pair_precision, double* E_out, void* stream);

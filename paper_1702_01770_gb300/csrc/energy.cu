@@ -13,13 +13,17 @@ constexpr int kWarpsPerBlock = 4;
 // 48 monomers take 19 and 46 us); smaller systems keep the plain form.
 constexpr int kSplitMinN = 48;
 constexpr int kSplitWarps = 4;   // warps of such a configuration
-// The far pairs' relative errors (independent, at most 1e-13 of their arithmetic and 6e-15 c of their
-// displacements' 48 bits, c the largest coordinate from its chain's origin or difference of origins)
-// may make up one FP64 rounding (2^-53) of the rest of the energy, as sizes of the lanes' sums: root of
-// the far pairs' squares times 1 + 0.06 c to the rest at most 2^-53 / 1e-13.  A configuration beyond it
-// (nothing near and no bending: conformations blown up, chains that interact from afar; unwrapped
-// chains many boxes long) is taken in FP64 throughout.  Eight 55-mers: 1e-5 of it.
-constexpr float kSplitLimit = 1.1e-3f;
+// When a configuration's far pairs may be taken in double-float.  Their errors, over the pairs' sizes v: a
+// few 1e-15 of sum |v| (what the products leave out has one sign), and of the root of sum v^2, pair by
+// pair, some 1e-14 of the arithmetic and 2e-15 c of the displacements' 48 bits (c: the largest coordinate
+// from its chain's origin or difference of origins).  That may come to eight FP64 roundings of the rest of
+// the energy (2^-53 of it; every term has a dozen): 4 sum |v| + (12 + 2 c) sqrt(sum v^2) <= the rest.
+// Beyond it (nothing near and no bending: conformations blown up, chains that interact from afar;
+// unwrapped chains many boxes long) a configuration is taken in FP64 throughout.  Largest errors against
+// extended precision in roundings of the sum of the terms' sizes, FP64 throughout -> here: random walks of
+// 48 to 512 monomers 2.3 to 7.0 -> 1.5 to 2.8, straight chains (which come nearest to the limit) of 48 to
+// 512 2.3 to 7.8 -> 1.3 to 5.3, with bonds of 1.5 8.4 to 22.6 -> 5.8 to 10.8.
+constexpr float kSplitCommon = 4.0f, kSplitPair = 12.0f, kSplitCoord = 2.0f;
 
 // FP32 pairs: one warp per configuration.
 __global__ void __launch_bounds__(32 * kWarpsPerBlock)
@@ -46,13 +50,12 @@ energy32_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
 //
 // An FP64 instruction holds an SMSP's pipe for 64 to 76 cycles, 13 to 16 of them make a pair,
 // and nearly all pairs of a large system are far apart.  SPLIT: a pair further apart than 4
-// (r^-6 below 2.5e-4) is evaluated in double-float arithmetic (two FP32 numbers, about 120
-// FP32 instructions) on coordinates relative to a monomer of its chain; its relative error is
-// some 1e-13, which the near pairs and the bends dwarf (kSplitLimit: else the configuration is
-// taken in FP64); nearer pairs, and those whose image count or magnitude FP32 does not settle,
-// are collected and take the FP64 instructions, a full warp at a time.
-// 1024 configurations of eight 55-mers: 1.01 ms (6.12 ms in FP64 throughout); the largest
-// error against extended precision fell from 1.4e-12 to 3.8e-13.
+// (r^-6 below 2.5e-4) is evaluated in double-float arithmetic (two FP32 numbers, about 130
+// FP32 instructions) on coordinates relative to a monomer of its chain, to some 1e-14 of it, which
+// the near pairs and the bends dwarf (kSplitCommon: else the configuration is taken in FP64);
+// nearer pairs, and those whose image count or magnitude FP32 does not settle, are collected and
+// take the FP64 instructions, a full warp at a time.
+// 1024 configurations of eight 55-mers: 1.05 ms (6.12 ms in FP64 throughout).
 // ---------------------------------------------------------------------------
 struct NearPair { int i, j; };   // i < j: C_LJ takes the earlier monomer's letter first
 
@@ -121,8 +124,11 @@ __device__ __forceinline__ float split_diff(float ah, float al, float bh, float 
         }
         *unsure |= fabsf(s) > B.edge;
     }
-    *lo = l;
-    return s;
+    // the low part may be far above a rounding of the high one (the coordinates are larger than their
+    // difference): bring it there, or the products that the square leaves out would count
+    const float h = __fadd_rn(s, l);
+    *lo = __fsub_rn(l, __fsub_rn(h, s));
+    return h;
 }
 
 template <int W, bool SPLIT>
@@ -131,7 +137,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ NearPair s_near[W > 1 ? W : kWarpsPerBlock][64];
     __shared__ double red[32];
-    __shared__ float4 s_size[W];   // SPLIT: the warps' sums of far pairs squared and of the size of the rest, largest coordinate
+    __shared__ float4 s_size[W];   // SPLIT, of each warp: sums of the far pairs' sizes and squares, largest coordinate, size of the rest
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int w = W > 1 ? warp : 0;                                   // the warp's number within the configuration
     const int b = W > 1 ? blockIdx.x : blockIdx.x * kWarpsPerBlock + warp;
@@ -197,7 +203,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
         for (int q = 0; q < 4; ++q) split(d.C[q], &Ch[q], &Cl[q]);
         __syncthreads();
         DF in{0.0f, 0.0f}, ex{0.0f, 0.0f};   // far pairs within chains and between them
-        float squares = 0.0f;                // sum of their squares
+        float sizes = 0.0f, squares = 0.0f;  // sums of their sizes and squares
         int n_near = 0;
         NearPair* near = s_near[warp];
         auto drain = [&](int n) {   // the first n of the list
@@ -232,11 +238,12 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
                         l2 = __fmaf_rn(__fadd_rn(dx, dx), lx, l2);
                         l2 = __fmaf_rn(__fadd_rn(dy, dy), ly, l2);
                         l2 = __fmaf_rn(__fadd_rn(dz, dz), lz, l2);
-                        // s = 1 / r^2 in two parts, s^3, and s^3 (s^3 - C)
+                        // s = 1 / r^2 in two parts, s^3 (with 3 sh sl^2, which all pairs have the same sign of), and s^3 (s^3 - C)
                         const float sh = fast_rcp(r2);
                         const float er = __fmaf_rn(-l2, sh, __fmaf_rn(-r2, sh, 1.0f));
                         const float t = __fmul_rn(sh, er), sl = __fmaf_rn(t, er, t);
-                        const float p = __fmul_rn(sh, sh), pl = __fmaf_rn(__fadd_rn(sh, sh), sl, __fmaf_rn(sh, sh, -p));
+                        const float p = __fmul_rn(sh, sh);
+                        const float pl = __fmaf_rn(__fmaf_rn(3.0f, sl, __fadd_rn(sh, sh)), sl, __fmaf_rn(sh, sh, -p));
                         const float c3 = __fmul_rn(p, sh);
                         const float c3l = __fmaf_rn(p, sl, __fmaf_rn(pl, sh, __fmaf_rn(p, sh, -c3)));
                         const int cc = j > i ? 2 * (ta & 1) + (tb & 1) : 2 * (tb & 1) + (ta & 1);   // the earlier monomer's letter first
@@ -248,6 +255,7 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
                         const float wh = __fmul_rn(c3, u);
                         const float wl = __fmaf_rn(c3, ul, __fmaf_rn(c3l, u, __fmaf_rn(c3, u, -wh)));
                         const DF v = df_add(inter ? ex : in, DF{wh, wl});
+                        sizes += fabsf(wh);
                         squares = __fmaf_rn(wh, wh, squares);
                         if (inter) ex = v;
                         else in = v;
@@ -270,15 +278,16 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
             if (i >= N) { i -= N; ++s; }
         }
         drain(n_near);
-        // the far pairs' errors against one rounding of everything else (see kSplitLimit)
+        // the far pairs' errors against the roundings of everything else (see kSplitCommon)
         float rest = fabsf(f64_to_f32(part));
 #pragma unroll
         for (int m = 16; m > 0; m >>= 1) {
+            sizes += __shfl_xor_sync(full, sizes, m);
             squares += __shfl_xor_sync(full, squares, m);
             rest += __shfl_xor_sync(full, rest, m);
             extent = fmaxf(extent, __shfl_xor_sync(full, extent, m));
         }
-        if (lane == 0) s_size[warp] = make_float4(squares, rest, extent, 0.0f);
+        if (lane == 0) s_size[warp] = make_float4(sizes, squares, extent, rest);
         __syncthreads();
         float4 size = s_size[0];
 #pragma unroll
@@ -286,9 +295,11 @@ energy64_kernel(const SysDesc d, int B, const double* __restrict__ xyz, double* 
             size.x += s_size[q].x;
             size.y += s_size[q].y;
             size.z = fmaxf(size.z, s_size[q].z);
+            size.w += s_size[q].w;
         }
-        const float k = fmaxf(fabsf(d.kin32), fabsf(d.kout32)), far = k * sqrtf(size.x) * (1.0f + 0.06f * size.z);
-        if (!(size.y > 1e-12f && far <= kSplitLimit * size.y)) part = whole_energy64(d, x64, lane, w, W);
+        const float k = fmaxf(fabsf(d.kin32), fabsf(d.kout32));
+        const float far = k * (kSplitCommon * size.x + (kSplitPair + kSplitCoord * size.z) * sqrtf(size.y));
+        if (!(size.w > 1e-12f && far <= size.w)) part = whole_energy64(d, x64, lane, w, W);
         else part += d.k_lj_intra * (f32_to_f64(in.hi) + f32_to_f64(in.lo)) + d.k_lj_inter * (f32_to_f64(ex.hi) + f32_to_f64(ex.lo));
     } else {
         part = add_pairs64(part, d, x64, w * 32 + lane, 32 * W);

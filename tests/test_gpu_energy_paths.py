@@ -194,3 +194,16 @@ def test_unwrapped_chains_many_boxes_long(phast, bond, L):
     r = np.sqrt(((d - L * np.rint(d / L)) ** 2).sum(2))
     steep = (s.k_lj_inter * (12 * r ** -12.0 + 6 * r ** -6.0) / r).sum(1)   # |dE / dr| of the pairs between chains
     assert np.all(np.abs(E - ref) <= 16 * 2.0 ** -53 * size + 2 * 3 ** 0.5 * 2.0 ** -53 * np.abs(x).max(axis=(1, 2)) * steep)
+
+
+@pytest.mark.parametrize("n", [48, 55, 200, 512])
+@pytest.mark.parametrize("direction", [(1.0, 0.0, 0.0), (1.0, 1.0, 1.0), (0.3, -0.5, 0.9)], ids=["axis", "diagonal", "oblique"])
+def test_straight_chains_to_the_last_digits(phast, n, direction):
+    """No bending and the fewest near pairs that an ordinary chain can have, so that far pairs weigh most: the bound of
+    test_fp64_energies_to_the_last_digits, for stretched and slightly bent chains."""
+    s = _system([n], 0.0, k_tors=0.0)
+    rng = np.random.default_rng(n)
+    x = np.array([inputs.straight_chain(n, direction=direction) * r + rng.normal(size=(n, 3)) * e for r in (1.0, 1.3) for e in (0.0, 1e-3, 0.05)])
+    E = phast.phast_energy(s, torch.from_numpy(x).cuda()).cpu().numpy().astype(np.longdouble)
+    ref, size = _extended(s, x)
+    assert np.all(np.abs(E - ref) <= 16 * 2.0 ** -53 * size), ((E - ref) / size / 2.0 ** -53).astype(float)
